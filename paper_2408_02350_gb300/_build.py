@@ -14,7 +14,7 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libbgk.so")
 LIB_DEBUG = os.path.join(HERE, "libbgk_debug.so")
-SOURCES = ["abi.cu", "nbr_stencil.cu", "step.cu", "chain.cu", "adjoint.cu", "manage.cu", "noalloc.cu", "peak.cu"]
+SOURCES = ["abi.cu", "nbr_stencil.cu", "step.cu", "transport_f64.cu", "chain.cu", "adjoint.cu", "manage.cu", "noalloc.cu", "peak.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"),
          "-I", CSRC]

@@ -181,6 +181,13 @@ int launch_transport_avg(const CaseView& cv, cudaStream_t s);
 int launch_relax_half(const CaseView& cv, cudaStream_t s);
 // FP32 warp-per-point transport + relaxation (used by the adjoint's forward recomputation)
 int launch_transport_fp32(const CaseView& cv, cudaStream_t s);
+// FP64 storage (transport_f64.cu): the transport of the step, of the sharded step and of the
+// second stage of the second-order step, and the in-place relaxations.
+int launch_transport_f64(const CaseView& cv, cudaStream_t s);
+int launch_transport_f64_shard(const CaseView& cv, cudaStream_t s);
+int launch_transport_f64_avg(const CaseView& cv, cudaStream_t s);
+int launch_relax_half_f64(const CaseView& cv, cudaStream_t s);
+int launch_shard_relax_f64(const CaseView& cv, cudaStream_t s);
 int launch_walls(const CaseView& cv, cudaStream_t s);
 // Batched (many cases, one launch each): FP32/BF16 storage, all cases of one dimension.
 int launch_transport_batch(const CaseView* d_cases, const int2* items, int n_items, int dim, int storage, int capmax,

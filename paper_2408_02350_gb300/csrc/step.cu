@@ -1,19 +1,16 @@
 // Per-step kernels of the meshfree BGK scheme (Sec. 3.2, 3.4.2, 5).
 //
-// k_transport: one CTA per interior point i; each thread owns NCH chunks of 4
-//   consecutive velocities.  The neighbour list and stencil of i are staged
-//   in shared memory; for every neighbour j the thread reads f_j for its
-//   velocities (16-byte loads, a warp reads 512 contiguous bytes per chunk)
-//   and accumulates
+// k_transport_wp, k_transport_mirror, k_transport_batch (FP32 arithmetic; FP64 storage:
+//   transport_f64.cu): one warp per interior point i.  The neighbour list and stencil of
+//   i are staged in shared memory; for every neighbour j each lane reads f_j for its
+//   velocities (16-byte loads) and accumulates
 //     m_ij(v) = sum_d min(c.P_d, 0),  acc += m_ij f_j,  sk += m_ij,
 //   with c = v - U_i^n (ALE) or v.  Since the upwind coefficient is
 //   K_ij = sum_d (c.P_d - |c.P_d|) = 2 m_ij, the transported value is
 //     f~_i = f_i - dt sum_j K_ij (f_j - f_i) = f_i - 2 dt (acc - sk f_i).
-//   The same CTA then sums the moments of f~_i over all velocities (warp
-//   shuffles, cross-warp totals in double by one thread), forms rho, U, T,
-//   tau and the Maxwellian, and writes f^{n+1} = (tau f~ + dt M)/(tau + dt)
-//   to the other buffer: one read of f_i, neighbour reads served mostly from
-//   L2, one write of f_i^{n+1}.
+//   The same warp then sums the moments of f~_i over all velocities, forms rho, U, T,
+//   tau and the Maxwellian, and writes f^{n+1} = (tau f~ + dt M)/(tau + dt) to the other
+//   buffer: one read of f_i, neighbour reads served mostly from L1 and L2, one write.
 // k_walls: one CTA per wall point; arriving velocities (v.n <= 0) get the WLS
 //   reconstruction from interior f^{n+1}; leaving velocities get
 //   rho_w M_w(v) with rho_w from zero net mass flux.
@@ -52,15 +49,6 @@ __device__ __forceinline__ void finish_moments(const double* tot, double wv, dou
   *rho = R * wv;
 }
 
-template <typename C>
-__device__ __forceinline__ C expc(C x);
-template <> __device__ __forceinline__ float expc<float>(float x) { return expf(x); }
-template <> __device__ __forceinline__ double expc<double>(double x) { return exp(x); }
-
-template <typename C> __device__ __forceinline__ C minc(C a, C b);
-template <> __device__ __forceinline__ float minc<float>(float a, float b) { return fminf(a, b); }
-template <> __device__ __forceinline__ double minc<double>(double a, double b) { return fmin(a, b); }
-
 // Sum NVAL per-thread values: warp shuffles in T, then thread 0 adds the warp
 // totals in double.  Result in out[] of every thread.
 template <int NVAL, typename T>
@@ -85,386 +73,6 @@ __device__ __forceinline__ void block_sum0(const T (&v)[NVAL], double (&out)[NVA
 #pragma unroll
   for (int q = 0; q < NVAL; ++q) out[q] = scratch[q * 32];
   __syncthreads();
-}
-
-// ---------------------------------------------------------------------------
-// transport + moments + relaxation
-// ---------------------------------------------------------------------------
-// Moments of f~_i from the raw sums tot, tau and the Maxwellian (one thread, FP64,
-// broadcast through shared memory), then f^{n+1} = (tau f~ + dt M)/(tau + dt) (RK = 1:
-// the exact relaxation over dt/2) for the thread's chunks, written to the output row.
-// vk0: first grid velocity of the row.
-template <typename S, typename C, int DIM, int NCH, int RK = 0>
-__device__ __forceinline__ void relax_cta(const CaseView& cv, const int i, const double (&tot)[DIM + 2],
-                                          const C (&ft)[NCH][DIM == 2 ? 2 : 1][4], const C* s_v, double* s_red,
-                                          const int vk0) {
-  constexpr int NC = DIM == 2 ? 2 : 1;
-  const int nv = cv.nv, NV = cv.NV, NVp = cv.NVp;
-  const int nchunk = NVp >> 2;
-  const int64_t rowlen = (int64_t)NC * NVp;
-  // moments, tau and relaxation coefficients (one thread, FP64), broadcast through shared memory
-  C* s_fin = reinterpret_cast<C*>(s_red + 6 * 32);  // past the slots block_sum0 uses (5 x 32)
-  if (threadIdx.x == 0) {
-    double rho, Un[3] = {0, 0, 0}, T;
-    const double wv = cv.wv;
-    finish_moments<DIM>(tot, wv, &rho, Un, &T);
-    double* mo = cv.mom + (int64_t)i * MOM_STRIDE;
-    mo[0] = rho; mo[1] = Un[0]; mo[2] = Un[1]; mo[3] = Un[2]; mo[4] = T;
-    double a = 1.0, b = 0.0, pref = 0.0, inv2T = 0.0;
-    if (!(rho > 0.0) || !(T > 0.0) || !isfinite(rho) || !isfinite(T)) {
-      set_status(cv.status, ST_NONFINITE);
-    } else if (cv.tau_mode != 2) {
-      const double pi = 3.14159265358979323846;
-      const double tau = cv.tau_mode == 1 ? sqrt(2.0 / pi) * cv.kn : sqrt(2.0 / pi) * cv.kn / (rho * sqrt(T));
-      if (RK == 1) {
-        a = exp(-0.5 * cv.dt / tau);
-        b = -expm1(-0.5 * cv.dt / tau);
-      } else {
-        a = tau / (tau + cv.dt);
-        b = cv.dt / (tau + cv.dt);
-      }
-      pref = DIM == 2 ? rho / (2.0 * pi * T) : rho / pow(2.0 * pi * T, 1.5);
-      inv2T = 1.0 / (2.0 * T);
-    }
-    s_fin[0] = (C)a; s_fin[1] = (C)b; s_fin[2] = (C)pref; s_fin[3] = (C)inv2T; s_fin[4] = (C)T;
-#pragma unroll
-    for (int d = 0; d < DIM; ++d) s_fin[5 + d] = (C)Un[d];
-  }
-  __syncthreads();
-  const C ca = s_fin[0], cb = s_fin[1], pref = s_fin[2], inv2T = s_fin[3], Tn = s_fin[4];
-  C Un[DIM];
-#pragma unroll
-  for (int d = 0; d < DIM; ++d) Un[d] = s_fin[5 + d];
-
-  S* fo = reinterpret_cast<S*>(cv.f_out) + (int64_t)i * rowlen;
-#pragma unroll
-  for (int q = 0; q < NCH; ++q) {
-    const int chunk = threadIdx.x + q * blockDim.x;
-    if (chunk < nchunk) {
-      C out[NC][4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int k = 4 * chunk + e;
-        if (k < NV) {
-          int kk = k + vk0;
-          C c2 = (C)0;
-#pragma unroll
-          for (int a = 0; a < DIM; ++a) {
-            const C d = s_v[kk % nv] - Un[a];
-            kk /= nv;
-            c2 += d * d;
-          }
-          const C M = pref * expc<C>(-c2 * inv2T);
-          out[0][e] = ca * ft[q][0][e] + cb * M;
-          if (NC == 2) out[NC - 1][e] = ca * ft[q][NC - 1][e] + cb * Tn * M;
-        } else {
-#pragma unroll
-          for (int c = 0; c < NC; ++c) out[c][e] = (C)0;
-        }
-      }
-#pragma unroll
-      for (int c = 0; c < NC; ++c) st4(fo + (int64_t)c * NVp + 4 * chunk, out[c]);
-    }
-  }
-}
-
-template <typename S, typename C, int DIM, int NCH, bool ALE, bool SH = false, bool AVG = false>
-__global__ void __launch_bounds__(256) k_transport(const CaseView cv) {
-  constexpr int NC = DIM == 2 ? 2 : 1;
-  constexpr int DD = DIM * DIM;
-  extern __shared__ __align__(16) unsigned char smem[];
-  double* s_red = reinterpret_cast<double*>(smem);
-  C* s_v = reinterpret_cast<C*>(smem + RED_BYTES);
-  int32_t* s_col = reinterpret_cast<int32_t*>(smem + RED_BYTES + NODE_BYTES);
-  C* s_P = reinterpret_cast<C*>(smem + RED_BYTES + NODE_BYTES + align16(sizeof(int32_t) * cv.cap));
-
-  const int i = cv.int_idx[blockIdx.x];
-  const int m = checked_count(cv.cnt[i], cv.cap, cv.status);
-  const int nv = cv.nv, NV = cv.NV, NVp = cv.NVp;
-  const int nchunk = NVp >> 2;
-  const int vk0 = SH ? cv.vk0 : 0;
-  {
-    const int32_t* col = cv.col + (int64_t)i * cv.cap;
-    const C* P = reinterpret_cast<const C*>(cv.P) + (int64_t)i * cv.cap * DD;
-    for (int t = threadIdx.x; t < m; t += blockDim.x) s_col[t] = checked_index(col[t], cv.n, i, cv.status);
-    for (int t = threadIdx.x; t < m * DD; t += blockDim.x) s_P[t] = P[t];
-    for (int t = threadIdx.x; t < nv; t += blockDim.x) s_v[t] = (C)cv.vnodes[t];
-  }
-  __syncthreads();
-
-  C U[DIM];
-#pragma unroll
-  for (int a = 0; a < DIM; ++a) U[a] = ALE ? (C)cv.mom[(int64_t)i * MOM_STRIDE + 1 + a] : (C)0;
-
-  // convective velocities c = v - U of this thread's velocities
-  C cvel[NCH][4][DIM];
-#pragma unroll
-  for (int q = 0; q < NCH; ++q) {
-    const int chunk = threadIdx.x + q * blockDim.x;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int k = 4 * chunk + e;
-      int kk = k < NV ? k + vk0 : 0;
-#pragma unroll
-      for (int a = 0; a < DIM; ++a) {
-        cvel[q][e][a] = k < NV ? s_v[kk % nv] - U[a] : (C)0;
-        kk /= nv;
-      }
-    }
-  }
-
-  C acc[NCH][NC][4], sk[NCH][4];
-#pragma unroll
-  for (int q = 0; q < NCH; ++q)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      sk[q][e] = (C)0;
-#pragma unroll
-      for (int c = 0; c < NC; ++c) acc[q][c][e] = (C)0;
-    }
-
-  const S* fbase = reinterpret_cast<const S*>(cv.f_in);
-  const int64_t rowlen = (int64_t)NC * NVp;
-  for (int s = 0; s < m; ++s) {
-    const int j = s_col[s];
-    C P[DD];
-#pragma unroll
-    for (int t = 0; t < DD; ++t) P[t] = s_P[s * DD + t];
-    const S* fj = fbase + (int64_t)j * rowlen;
-#pragma unroll
-    for (int q = 0; q < NCH; ++q) {
-      const int chunk = threadIdx.x + q * blockDim.x;
-      if (chunk < nchunk) {
-        C fv[NC][4];
-#pragma unroll
-        for (int c = 0; c < NC; ++c) ld4(fj + (int64_t)c * NVp + 4 * chunk, fv[c]);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          C mk = (C)0;
-#pragma unroll
-          for (int d = 0; d < DIM; ++d) {
-            C p = cvel[q][e][0] * P[d * DIM + 0];
-#pragma unroll
-            for (int a = 1; a < DIM; ++a) p += cvel[q][e][a] * P[d * DIM + a];
-            mk += minc(p, (C)0);
-          }
-          sk[q][e] += mk;
-#pragma unroll
-          for (int c = 0; c < NC; ++c) acc[q][c][e] += mk * fv[c][e];
-        }
-      }
-    }
-  }
-
-  // f~ = f_i - 2 dt (acc - sk f_i) and one-pass raw moment sums
-  const S* fi = fbase + (int64_t)i * rowlen;
-  const C two_dt = (C)(2.0 * cv.dt);
-  C ft[NCH][NC][4];
-  C part[DIM + 2];
-#pragma unroll
-  for (int t = 0; t < DIM + 2; ++t) part[t] = (C)0;
-#pragma unroll
-  for (int q = 0; q < NCH; ++q) {
-    const int chunk = threadIdx.x + q * blockDim.x;
-    if (chunk < nchunk) {
-      C fiv[NC][4], fav[NC][4];
-#pragma unroll
-      for (int c = 0; c < NC; ++c) ld4(fi + (int64_t)c * NVp + 4 * chunk, fiv[c]);
-      if (AVG) {
-        const S* fa = reinterpret_cast<const S*>(cv.f_avg) + (int64_t)i * rowlen;
-#pragma unroll
-        for (int c = 0; c < NC; ++c) ld4(fa + (int64_t)c * NVp + 4 * chunk, fav[c]);
-      }
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-#pragma unroll
-        for (int c = 0; c < NC; ++c) ft[q][c][e] = fiv[c][e] - two_dt * (acc[q][c][e] - sk[q][e] * fiv[c][e]);
-        if (AVG) {
-#pragma unroll
-          for (int c = 0; c < NC; ++c) ft[q][c][e] = (C)0.5 * (ft[q][c][e] + fav[c][e]);
-        }
-        const int k = 4 * chunk + e;
-        if (k < NV) {
-          int kk = k + vk0;
-          C v2 = (C)0;
-          const C g = ft[q][0][e];
-          part[0] += g;
-#pragma unroll
-          for (int a = 0; a < DIM; ++a) {
-            const C va = s_v[kk % nv];
-            kk /= nv;
-            part[1 + a] += va * g;
-            v2 += va * va;
-          }
-          part[DIM + 1] += v2 * g;
-          if (NC == 2) part[DIM + 1] += ft[q][NC - 1][e];
-        }
-      }
-    } else {
-#pragma unroll
-      for (int e = 0; e < 4; ++e)
-#pragma unroll
-        for (int c = 0; c < NC; ++c) ft[q][c][e] = (C)0;
-    }
-  }
-  double tot[DIM + 2];
-  block_sum0<DIM + 2, C>(part, tot, s_red);
-
-  if constexpr (SH) {
-    // sharded step: the slab's sums to the exchange buffer, f~ to the output row
-    if (threadIdx.x == 0) {
-#pragma unroll
-      for (int q = 0; q < DIM + 2; ++q) cv.xs[(int64_t)i * (DIM + 2) + q] = tot[q];
-    }
-    S* fo = reinterpret_cast<S*>(cv.f_out) + (int64_t)i * rowlen;
-#pragma unroll
-    for (int q = 0; q < NCH; ++q) {
-      const int chunk = threadIdx.x + q * blockDim.x;
-      if (chunk < nchunk) {
-#pragma unroll
-        for (int c = 0; c < NC; ++c) st4(fo + (int64_t)c * NVp + 4 * chunk, ft[q][c]);
-      }
-    }
-  } else {
-    relax_cta<S, C, DIM, NCH, AVG ? 1 : 0>(cv, i, tot, ft, s_v, s_red, 0);
-  }
-}
-
-template <typename S, typename C, int DIM, int NCH, bool SH = false, bool AVG = false>
-static void launch_transport_t(const CaseView& cv, int threads, size_t smem, cudaStream_t s) {
-  if (AVG) {
-    // the second-order step is for fixed points
-    auto k = k_transport<S, C, DIM, NCH, false, false, true>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k<<<cv.n_int, threads, smem, s>>>(cv);
-  } else if (cv.ale) {
-    auto k = k_transport<S, C, DIM, NCH, true, SH>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k<<<cv.n_int, threads, smem, s>>>(cv);
-  } else {
-    auto k = k_transport<S, C, DIM, NCH, false, SH>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k<<<cv.n_int, threads, smem, s>>>(cv);
-  }
-}
-
-// Sharded step, FP64 storage: one CTA per interior point (the launch shape of
-// k_transport) relaxes f~ in the output row with the moments of the summed sums.
-template <typename S, typename C, int DIM, int NCH>
-__global__ void __launch_bounds__(256) k_shard_relax_cta(const CaseView cv) {
-  constexpr int NC = DIM == 2 ? 2 : 1;
-  __shared__ double s_red[8 * 32];
-  __shared__ C s_v[64];
-  const int i = cv.int_idx[blockIdx.x];
-  const int NVp = cv.NVp, nchunk = NVp >> 2;
-  for (int t = threadIdx.x; t < cv.nv; t += blockDim.x) s_v[t] = (C)cv.vnodes[t];
-  const S* fo = reinterpret_cast<const S*>(cv.f_out) + (int64_t)i * NC * NVp;
-  C ft[NCH][NC][4];
-#pragma unroll
-  for (int q = 0; q < NCH; ++q) {
-    const int chunk = threadIdx.x + q * blockDim.x;
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      if (chunk < nchunk) {
-        ld4(fo + (int64_t)c * NVp + 4 * chunk, ft[q][c]);
-      } else {
-#pragma unroll
-        for (int e = 0; e < 4; ++e) ft[q][c][e] = (C)0;
-      }
-    }
-  }
-  double tot[DIM + 2];
-#pragma unroll
-  for (int q = 0; q < DIM + 2; ++q) tot[q] = cv.xs[(int64_t)i * (DIM + 2) + q];
-  __syncthreads();
-  relax_cta<S, C, DIM, NCH>(cv, i, tot, ft, s_v, s_red, cv.vk0);
-}
-
-// CTA shape of the FP64 transport: NCH chunks of 4 velocities per thread, at most 256 threads.
-static inline void cta_shape(int NVp, int* nch, int* threads) {
-  const int nchunk = NVp / 4;
-  int q = 1;
-  while ((nchunk + q - 1) / q > 256) q *= 2;
-  *nch = q;
-  *threads = (((nchunk + q - 1) / q) + 31) / 32 * 32;
-}
-
-template <typename S, typename C, int DIM, bool SH = false, bool AVG = false>
-static void launch_transport_d(const CaseView& cv, cudaStream_t s) {
-  int nch, threads;
-  cta_shape(cv.NVp, &nch, &threads);
-  const size_t smem = RED_BYTES + NODE_BYTES + align16(sizeof(int32_t) * cv.cap) + sizeof(C) * cv.cap * DIM * DIM;
-  switch (nch) {
-    case 1: launch_transport_t<S, C, DIM, 1, SH, AVG>(cv, threads, smem, s); break;
-    case 2: launch_transport_t<S, C, DIM, 2, SH, AVG>(cv, threads, smem, s); break;
-    case 4: launch_transport_t<S, C, DIM, 4, SH, AVG>(cv, threads, smem, s); break;
-    default: launch_transport_t<S, C, DIM, 8, SH, AVG>(cv, threads, smem, s); break;
-  }
-}
-
-// Second-order step, FP64 storage: the exact relaxation over dt/2 of the output row of
-// each interior point in place, with the moments of that row (one CTA per point).
-template <typename S, typename C, int DIM, int NCH>
-__global__ void __launch_bounds__(256) k_relax_half_cta(const CaseView cv) {
-  constexpr int NC = DIM == 2 ? 2 : 1;
-  __shared__ double s_red[8 * 32];
-  __shared__ C s_v[64];
-  const int i = cv.int_idx[blockIdx.x];
-  const int nv = cv.nv, NV = cv.NV, NVp = cv.NVp, nchunk = NVp >> 2;
-  for (int t = threadIdx.x; t < nv; t += blockDim.x) s_v[t] = (C)cv.vnodes[t];
-  __syncthreads();
-  const S* fo = reinterpret_cast<const S*>(cv.f_out) + (int64_t)i * NC * NVp;
-  C ft[NCH][NC][4];
-  C part[DIM + 2];
-#pragma unroll
-  for (int t = 0; t < DIM + 2; ++t) part[t] = (C)0;
-#pragma unroll
-  for (int q = 0; q < NCH; ++q) {
-    const int chunk = threadIdx.x + q * blockDim.x;
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      if (chunk < nchunk) {
-        ld4(fo + (int64_t)c * NVp + 4 * chunk, ft[q][c]);
-      } else {
-#pragma unroll
-        for (int e = 0; e < 4; ++e) ft[q][c][e] = (C)0;
-      }
-    }
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int k = 4 * chunk + e;
-      if (chunk < nchunk && k < NV) {
-        int kk = k;
-        C v2 = (C)0;
-        const C g = ft[q][0][e];
-        part[0] += g;
-#pragma unroll
-        for (int a = 0; a < DIM; ++a) {
-          const C va = s_v[kk % nv];
-          kk /= nv;
-          part[1 + a] += va * g;
-          v2 += va * va;
-        }
-        part[DIM + 1] += v2 * g;
-        if (NC == 2) part[DIM + 1] += ft[q][NC - 1][e];
-      }
-    }
-  }
-  double tot[DIM + 2];
-  block_sum0<DIM + 2, C>(part, tot, s_red);
-  relax_cta<S, C, DIM, NCH, 1>(cv, i, tot, ft, s_v, s_red, 0);
-}
-
-template <typename S, typename C, int DIM>
-static void launch_shard_relax_d(const CaseView& cv, cudaStream_t s) {
-  int nch, threads;
-  cta_shape(cv.NVp, &nch, &threads);
-  switch (nch) {
-    case 1: k_shard_relax_cta<S, C, DIM, 1><<<cv.n_int, threads, 0, s>>>(cv); break;
-    case 2: k_shard_relax_cta<S, C, DIM, 2><<<cv.n_int, threads, 0, s>>>(cv); break;
-    case 4: k_shard_relax_cta<S, C, DIM, 4><<<cv.n_int, threads, 0, s>>>(cv); break;
-    default: k_shard_relax_cta<S, C, DIM, 8><<<cv.n_int, threads, 0, s>>>(cv); break;
-  }
 }
 
 // Shared memory of the warp-per-point kernels with W warps: velocity nodes, lists,
@@ -742,28 +350,15 @@ static void launch_transport_avg_wp(const CaseView& cv, cudaStream_t s) {
 
 int launch_transport_avg(const CaseView& cv, cudaStream_t s) {
   if (cv.n_int == 0) return 0;
+  if (cv.storage == 0) return launch_transport_f64_avg(cv, s);
   if (cv.dim == 2) {
-    if (cv.storage == 0) launch_transport_d<double, double, 2, false, true>(cv, s);
-    else if (cv.storage == 1) launch_transport_avg_wp<float, 2>(cv, s);
+    if (cv.storage == 1) launch_transport_avg_wp<float, 2>(cv, s);
     else launch_transport_avg_wp<__nv_bfloat16, 2>(cv, s);
   } else {
-    if (cv.storage == 0) launch_transport_d<double, double, 3, false, true>(cv, s);
-    else if (cv.storage == 1) launch_transport_avg_wp<float, 3>(cv, s);
+    if (cv.storage == 1) launch_transport_avg_wp<float, 3>(cv, s);
     else launch_transport_avg_wp<__nv_bfloat16, 3>(cv, s);
   }
   return 1;
-}
-
-template <typename S, typename C, int DIM>
-static void launch_relax_half_d(const CaseView& cv, cudaStream_t s) {
-  int nch, threads;
-  cta_shape(cv.NVp, &nch, &threads);
-  switch (nch) {
-    case 1: k_relax_half_cta<S, C, DIM, 1><<<cv.n_int, threads, 0, s>>>(cv); break;
-    case 2: k_relax_half_cta<S, C, DIM, 2><<<cv.n_int, threads, 0, s>>>(cv); break;
-    case 4: k_relax_half_cta<S, C, DIM, 4><<<cv.n_int, threads, 0, s>>>(cv); break;
-    default: k_relax_half_cta<S, C, DIM, 8><<<cv.n_int, threads, 0, s>>>(cv); break;
-  }
 }
 
 template <typename S, int DIM>
@@ -775,13 +370,12 @@ static void launch_relax_half_wp(const CaseView& cv, cudaStream_t s) {
 
 int launch_relax_half(const CaseView& cv, cudaStream_t s) {
   if (cv.n_int == 0 || cv.tau_mode == 2) return 0;
+  if (cv.storage == 0) return launch_relax_half_f64(cv, s);
   if (cv.dim == 2) {
-    if (cv.storage == 0) launch_relax_half_d<double, double, 2>(cv, s);
-    else if (cv.storage == 1) launch_relax_half_wp<float, 2>(cv, s);
+    if (cv.storage == 1) launch_relax_half_wp<float, 2>(cv, s);
     else launch_relax_half_wp<__nv_bfloat16, 2>(cv, s);
   } else {
-    if (cv.storage == 0) launch_relax_half_d<double, double, 3>(cv, s);
-    else if (cv.storage == 1) launch_relax_half_wp<float, 3>(cv, s);
+    if (cv.storage == 1) launch_relax_half_wp<float, 3>(cv, s);
     else launch_relax_half_wp<__nv_bfloat16, 3>(cv, s);
   }
   return 1;
@@ -789,13 +383,12 @@ int launch_relax_half(const CaseView& cv, cudaStream_t s) {
 
 int launch_transport(const CaseView& cv, cudaStream_t s) {
   if (cv.n_int == 0) return 0;
+  if (cv.storage == 0) return launch_transport_f64(cv, s);
   if (cv.dim == 2) {
-    if (cv.storage == 0) launch_transport_d<double, double, 2>(cv, s);
-    else if (cv.storage == 1) launch_transport_wp<float, 2>(cv, s);
+    if (cv.storage == 1) launch_transport_wp<float, 2>(cv, s);
     else launch_transport_wp<__nv_bfloat16, 2>(cv, s);
   } else {
-    if (cv.storage == 0) launch_transport_d<double, double, 3>(cv, s);
-    else if (cv.storage == 1) launch_transport_wp<float, 3>(cv, s);
+    if (cv.storage == 1) launch_transport_wp<float, 3>(cv, s);
     else launch_transport_wp<__nv_bfloat16, 3>(cv, s);
   }
   return 1;
@@ -1590,13 +1183,12 @@ static void launch_shard_transport_wp(const CaseView& cv, cudaStream_t s) {
 
 int launch_shard_transport(const CaseView& cv, cudaStream_t s) {
   if (cv.n_int == 0) return 0;
+  if (cv.storage == 0) return launch_transport_f64_shard(cv, s);
   if (cv.dim == 2) {
-    if (cv.storage == 0) launch_transport_d<double, double, 2, true>(cv, s);
-    else if (cv.storage == 1) launch_shard_transport_wp<float, 2>(cv, s);
+    if (cv.storage == 1) launch_shard_transport_wp<float, 2>(cv, s);
     else launch_shard_transport_wp<__nv_bfloat16, 2>(cv, s);
   } else {
-    if (cv.storage == 0) launch_transport_d<double, double, 3, true>(cv, s);
-    else if (cv.storage == 1) launch_shard_transport_wp<float, 3>(cv, s);
+    if (cv.storage == 1) launch_shard_transport_wp<float, 3>(cv, s);
     else launch_shard_transport_wp<__nv_bfloat16, 3>(cv, s);
   }
   return 1;
@@ -1611,13 +1203,12 @@ static void launch_shard_relax_wp(const CaseView& cv, cudaStream_t s) {
 
 int launch_shard_relax(const CaseView& cv, cudaStream_t s) {
   if (cv.n_int == 0) return 0;
+  if (cv.storage == 0) return launch_shard_relax_f64(cv, s);
   if (cv.dim == 2) {
-    if (cv.storage == 0) launch_shard_relax_d<double, double, 2>(cv, s);
-    else if (cv.storage == 1) launch_shard_relax_wp<float, 2>(cv, s);
+    if (cv.storage == 1) launch_shard_relax_wp<float, 2>(cv, s);
     else launch_shard_relax_wp<__nv_bfloat16, 2>(cv, s);
   } else {
-    if (cv.storage == 0) launch_shard_relax_d<double, double, 3>(cv, s);
-    else if (cv.storage == 1) launch_shard_relax_wp<float, 3>(cv, s);
+    if (cv.storage == 1) launch_shard_relax_wp<float, 3>(cv, s);
     else launch_shard_relax_wp<__nv_bfloat16, 3>(cv, s);
   }
   return 1;
