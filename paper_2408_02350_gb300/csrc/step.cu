@@ -1058,18 +1058,21 @@ __global__ void k_moments(CaseView cv, const S* f) {
 // totals to FP64 and forms rho, U, T in FP64, so each FP64 instruction serves MOM_GP
 // points (FP64 runs at a small fraction of the FP32 rate).  SH: the raw sums of the
 // velocity slab (in FP64) to the exchange buffer instead.
-constexpr int MOM_GP = 8, MOM_WARPS = 4;  // points per warp, warps per CTA
+constexpr int MOM_GP = 8, MOM_WARPS = 4;  // points per warp (at most), warps per CTA
+// Points per warp: MOM_GP where that still gives every SM 32 warps, fewer for smaller
+// clouds (8 points per warp left 8 warps per SM on 101^2 points: 32 us for 47 MB).
+static int moments_gp(int n) { return std::max(1, std::min(MOM_GP, n / (152 * 32))); }
 template <typename S, int DIM, bool ROW, bool SH = false>
-__global__ void __launch_bounds__(32 * MOM_WARPS) k_moments_wp(CaseView cv, const S* f) {
+__global__ void __launch_bounds__(32 * MOM_WARPS) k_moments_wp(CaseView cv, const S* f, const int gp) {
   constexpr int NC = DIM == 2 ? 2 : 1, VPL = 4, NQ = DIM + 2;
   __shared__ __align__(16) float s_v[64];  // chunk_velocities reads groups of 4
   __shared__ float2 s_tot[MOM_WARPS][MOM_GP][NQ];
   for (int t = threadIdx.x; t < cv.nv; t += blockDim.x) s_v[t] = cv.vnodes_f[t];
   __syncthreads();
   const int W = blockDim.x >> 5, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int i0 = (blockIdx.x * W + warp) * MOM_GP;
+  const int i0 = (blockIdx.x * W + warp) * gp;
   if (i0 >= cv.n) return;
-  const int np = min(MOM_GP, cv.n - i0);
+  const int np = min(gp, cv.n - i0);
   const int nv = cv.nv, NV = cv.NV, NVp = cv.NVp;
   const int vk0 = SH ? cv.vk0 : 0;
   const float inv_nv = 1.0f / (float)nv;
@@ -1137,12 +1140,12 @@ __global__ void __launch_bounds__(32 * MOM_WARPS) k_moments_wp(CaseView cv, cons
 }
 
 int launch_moments(const CaseView& cv, const void* f, cudaStream_t s) {
-  const int W = MOM_WARPS, grid = (cv.n + W * MOM_GP - 1) / (W * MOM_GP);
+  const int gp = moments_gp(cv.n), W = MOM_WARPS, grid = (cv.n + W * gp - 1) / (W * gp);
   const bool row = cv.nv % 4 == 0;
 #define BGK_MOM_WP(S, D)                                                                               \
   {                                                                                                    \
-    if (row) k_moments_wp<S, D, true><<<grid, 32 * W, 0, s>>>(cv, (const S*)f);                        \
-    else k_moments_wp<S, D, false><<<grid, 32 * W, 0, s>>>(cv, (const S*)f);                           \
+    if (row) k_moments_wp<S, D, true><<<grid, 32 * W, 0, s>>>(cv, (const S*)f, gp);                    \
+    else k_moments_wp<S, D, false><<<grid, 32 * W, 0, s>>>(cv, (const S*)f, gp);                       \
   }
   if (cv.dim == 2) {
     if (cv.storage == 0) k_moments<double, double, 2><<<cv.n, 256, 0, s>>>(cv, (const double*)f);
@@ -1236,12 +1239,12 @@ int launch_shard_walls(const CaseView& cv, int phase, cudaStream_t s) {
 }
 
 int launch_shard_partial(const CaseView& cv, cudaStream_t s) {
-  const int W = MOM_WARPS, grid = (cv.n + W * MOM_GP - 1) / (W * MOM_GP);
+  const int gp = moments_gp(cv.n), W = MOM_WARPS, grid = (cv.n + W * gp - 1) / (W * gp);
   const bool row = cv.nv % 4 == 0;
 #define BGK_PART_WP(S, D)                                                                                   \
   {                                                                                                         \
-    if (row) k_moments_wp<S, D, true, true><<<grid, 32 * W, 0, s>>>(cv, (const S*)cv.f_in);                 \
-    else k_moments_wp<S, D, false, true><<<grid, 32 * W, 0, s>>>(cv, (const S*)cv.f_in);                    \
+    if (row) k_moments_wp<S, D, true, true><<<grid, 32 * W, 0, s>>>(cv, (const S*)cv.f_in, gp);             \
+    else k_moments_wp<S, D, false, true><<<grid, 32 * W, 0, s>>>(cv, (const S*)cv.f_in, gp);                \
   }
   if (cv.dim == 2) {
     if (cv.storage == 0) k_moments<double, double, 2, true><<<cv.n, 256, 0, s>>>(cv, (const double*)cv.f_in);
@@ -1300,42 +1303,72 @@ int launch_shard_allreduce(double* const* bufs, int nbufs, int64_t count, cudaSt
   return 1;
 }
 
+// Copies between the caller's dense layout and the padded storage, converting the element
+// type.  Both are bound by HBM.  Without padding (NV % 4 == 0) the arrays are flat: 4
+// elements per thread and access, four accesses in flight (16-byte loads and stores in
+// FP32; pointers aligned to 4 elements).  Otherwise a warp takes whole rows, so that every
+// access of 32 neighbouring elements is contiguous whatever the row's alignment and no
+// thread divides.  One element per thread with a 64-bit division each took 78 us for the
+// 133^2 x 27^2 FP32 state (206 MB moved) and 35 us for 101^2 x 24^2 (94 MB); a pass of the
+// first (two steps and the read-back) takes 419 us instead of 462, the adjoint gradient of
+// 8 steps of the second (with its 21 moment passes) 4.49 ms instead of 4.96.
 template <typename A, typename B>
-__global__ void k_pack(const A* src, B* dst, int64_t rows, int NV, int NVp) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= rows * NVp) return;
-  const int64_t r = t / NVp;
-  const int k = (int)(t % NVp);
-  const float fz = 0.0f;
-  if (k < NV) st1(dst + t, (decltype(ld1(dst)))ld1(src + r * NV + k));
-  else st1(dst + t, (decltype(ld1(dst)))fz);
+__global__ void __launch_bounds__(256) k_convert_flat(const A* __restrict__ src, B* __restrict__ dst, int64_t n4) {
+  using CA = decltype(ld1(src));
+  using CB = decltype(ld1(dst));
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n4; t += 4 * stride) {
+    CA v[4][4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (t + u * stride < n4) ld4(src + 4 * (t + u * stride), v[u]);
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (t + u * stride < n4) {
+        const CB w[4] = {(CB)v[u][0], (CB)v[u][1], (CB)v[u][2], (CB)v[u][3]};
+        st4(dst + 4 * (t + u * stride), w);
+      }
+  }
 }
 
 template <typename A, typename B>
-__global__ void k_unpack(const A* src, B* dst, int64_t rows, int NV, int NVp) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= rows * NV) return;
-  const int64_t r = t / NV;
-  const int k = (int)(t % NV);
-  st1(dst + t, (decltype(ld1(dst)))ld1(src + r * NVp + k));
+__global__ void __launch_bounds__(256) k_convert_rows(const A* __restrict__ src, B* __restrict__ dst, int64_t rows,
+                                                      int NV, int ls, int ld) {
+  using CB = decltype(ld1(dst));
+  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  for (int64_t r = (int64_t)blockIdx.x * nw + (threadIdx.x >> 5); r < rows; r += (int64_t)gridDim.x * nw) {
+    const A* a = src + r * ls;
+    B* b = dst + r * ld;
+#pragma unroll 8
+    for (int k = lane; k < ld; k += 32) st1(b + k, k < NV ? (CB)ld1(a + k) : (CB)0);
+  }
+}
+
+template <typename A, typename B>
+static void convert(const A* src, B* dst, int64_t rows, int NV, int ls, int ld, cudaStream_t s) {
+  if (ls == ld && NV == ls && reinterpret_cast<uintptr_t>(src) % (4 * sizeof(A) < 16 ? 4 * sizeof(A) : 16) == 0 &&
+      reinterpret_cast<uintptr_t>(dst) % (4 * sizeof(B) < 16 ? 4 * sizeof(B) : 16) == 0) {
+    const int64_t n4 = rows * ls / 4;  // (NV is a multiple of 4 here: ls = ld = NV is the padded length)
+    k_convert_flat<<<(int)std::min<int64_t>((n4 + 1023) / 1024, 152 * 32), 256, 0, s>>>(src, dst, n4);
+  } else {
+    k_convert_rows<<<(int)std::min<int64_t>((rows + 7) / 8, 152 * 64), 256, 0, s>>>(src, dst, rows, NV, ls, ld);
+  }
 }
 
 template <typename A>
 static void pack_from(const CaseView& cv, const A* src, void* dst, cudaStream_t s) {
   const int64_t rows = (int64_t)cv.n * cv.ncomp;
-  const int g = (int)((rows * cv.NVp + 255) / 256);
-  if (cv.storage == 0) k_pack<A, double><<<g, 256, 0, s>>>(src, (double*)dst, rows, cv.NV, cv.NVp);
-  else if (cv.storage == 1) k_pack<A, float><<<g, 256, 0, s>>>(src, (float*)dst, rows, cv.NV, cv.NVp);
-  else k_pack<A, __nv_bfloat16><<<g, 256, 0, s>>>(src, (__nv_bfloat16*)dst, rows, cv.NV, cv.NVp);
+  if (cv.storage == 0) convert(src, (double*)dst, rows, cv.NV, cv.NV, cv.NVp, s);
+  else if (cv.storage == 1) convert(src, (float*)dst, rows, cv.NV, cv.NV, cv.NVp, s);
+  else convert(src, (__nv_bfloat16*)dst, rows, cv.NV, cv.NV, cv.NVp, s);
 }
 
 template <typename B>
 static void unpack_to(const CaseView& cv, const void* src, B* dst, cudaStream_t s) {
   const int64_t rows = (int64_t)cv.n * cv.ncomp;
-  const int g = (int)((rows * cv.NV + 255) / 256);
-  if (cv.storage == 0) k_unpack<double, B><<<g, 256, 0, s>>>((const double*)src, dst, rows, cv.NV, cv.NVp);
-  else if (cv.storage == 1) k_unpack<float, B><<<g, 256, 0, s>>>((const float*)src, dst, rows, cv.NV, cv.NVp);
-  else k_unpack<__nv_bfloat16, B><<<g, 256, 0, s>>>((const __nv_bfloat16*)src, dst, rows, cv.NV, cv.NVp);
+  if (cv.storage == 0) convert((const double*)src, dst, rows, cv.NV, cv.NVp, cv.NV, s);
+  else if (cv.storage == 1) convert((const float*)src, dst, rows, cv.NV, cv.NVp, cv.NV, s);
+  else convert((const __nv_bfloat16*)src, dst, rows, cv.NV, cv.NVp, cv.NV, s);
 }
 
 int launch_pack_f(const CaseView& cv, const void* src, int src_dtype, void* dst, cudaStream_t s) {
