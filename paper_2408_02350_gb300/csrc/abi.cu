@@ -394,6 +394,12 @@ int move_and_prebuild(bgk_ctx* ctx, CaseHost& c, cudaStream_t s) {
     ctx->launches += k;
     CKL(ctx);
     if ((st = timed_end(ctx, e, q))) return st;
+    if (nx.wls_order == 2) {
+      if ((st = timed_begin(ctx, K_STENCIL, q, &e))) return st;
+      ctx->launches += launch_stencils(nx, q, 1);
+      CKL(ctx);
+      if ((st = timed_end(ctx, e, q))) return st;
+    }
   } else {
     if ((st = timed_begin(ctx, K_MOVE, q, &e))) return st;
     ctx->launches += launch_move(c.cv, q);

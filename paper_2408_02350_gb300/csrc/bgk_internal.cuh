@@ -147,8 +147,8 @@ int launch_manage_apply(const CaseView& cv, int64_t cap_n, const int32_t* nn, co
 // ALE with a skin: rebuild the candidate lists if a point moved too far, then filter them.
 int launch_neighbours_skin(const CaseView& cv, cudaStream_t s);
 // ALE with a skin, FP32/BF16 storage: motion, candidate rebuild when due, filter and
-// interior stencils of the list set in cv as one cooperative launch (grid size cached
-// in *grid_cache); returns 1, or -1 when the cooperative launch is unavailable.  A grid
+// interior stencils (the linear fit; the second-order fit is launched after it) of the
+// list set in cv as one cooperative launch (grid size cached in *grid_cache); returns 1, or -1 when the cooperative launch is unavailable.  A grid
 // barrier waits at most max_spins polls (0: about a second), then the kernel records
 // ST_TIMEOUT and its CTAs return.
 bool chain_eligible(const CaseView& cv);

@@ -129,6 +129,7 @@ __global__ void __launch_bounds__(CHAIN_THREADS) k_chain(CaseView cv, double thr
     const bool in = i < cv.n;
     filter_group_point<DIM>(cv, in ? i : 0, in, lane, lo, hi);
     __syncwarp();
+    if (cv.wls_order == 2) continue;  // the second-order fit follows in a launch of its own
     const bool valid = in && cv.kind[i] == 0;
     stencil_grp_point<DIM, 4>(cv, valid ? i : 0, valid, lane & 3);
   }
@@ -144,7 +145,7 @@ void bounds(int dim, double r, float* lo, float* hi) {
 
 }  // namespace
 
-bool chain_eligible(const CaseView& cv) { return cv.ale && cv.sk && cv.storage != 0 && cv.wls_order != 2; }
+bool chain_eligible(const CaseView& cv) { return cv.ale && cv.sk && cv.storage != 0; }
 
 // CTAs per SM of the cooperative launch (0: as many as fit, 5 at 48 registers).  The
 // kernel runs beside the wall kernel; with fewer CTAs the two share the SMs instead of

@@ -160,7 +160,7 @@ __device__ bool solve_e0(double (&B)[M][M], double (&z)[M]) {
 }
 
 // Interior stencil of the second-order Taylor fit (Sec. 3.4.1, higher-order
-// approximation), FP64, one thread per point: basis b_j = (dr, dr_a dr_b for a <= b,
+// approximation) in 3D, FP64, one thread per point: basis b_j = (dr, dr_a dr_b for a <= b,
 // halved on the diagonal), B = sum_j w_j b_j b_j^T (MQ x MQ, MQ = dim + dim (dim + 1) / 2),
 // G = the first dim columns of B^-1 by Gauss-Jordan elimination with partial pivoting
 // on [B | e_0 .. e_{dim-1}] (B is symmetric, so they are its gradient rows), coef_j =
@@ -174,10 +174,10 @@ __device__ __forceinline__ void quad_basis_d(const double* xi, const double* xj,
     for (int c = a; c < DIM; ++c) b[k++] = a == c ? 0.5 * dr[a] * dr[a] : dr[a] * dr[c];
 }
 
-template <typename C, int DIM>
+template <typename C>
 __device__ void quad_stencil_point(const CaseView& cv, const int i, const double* xi, const int32_t* row,
                                    const int m, C* P) {
-  constexpr int MQ = DIM + DIM * (DIM + 1) / 2;
+  constexpr int DIM = 3, MQ = DIM + DIM * (DIM + 1) / 2;
   const double nah2 = -cv.alpha, hh = cv.h * cv.h;
   double B[MQ][MQ + DIM];
   for (int a = 0; a < MQ; ++a)
@@ -229,25 +229,204 @@ __device__ void quad_stencil_point(const CaseView& cv, const int i, const double
       coef[a] = w * acc;
     }
     const double r = sqrt(r2);
-    double E[DIM][DIM];  // rows n, t(, b)
-    if constexpr (DIM == 2) {
-      const double nx = dr[0] / r, ny = dr[1] / r;
-      E[0][0] = nx; E[0][1] = ny;
-      E[1][0] = -ny; E[1][1] = nx;
-    } else {
-      const double rxy = sqrt(dr[0] * dr[0] + dr[1] * dr[1]);
-      const double cphi = rxy > 0.0 ? dr[0] / rxy : 1.0, sphi = rxy > 0.0 ? dr[1] / rxy : 0.0;
-      const double cth = dr[2] / r, sth = rxy / r;
-      E[0][0] = dr[0] / r; E[0][1] = dr[1] / r; E[0][2] = dr[2] / r;
-      E[1][0] = cth * cphi; E[1][1] = cth * sphi; E[1][2] = -sth;
-      E[2][0] = -sphi; E[2][1] = cphi; E[2][2] = 0.0;
-    }
+    double E[DIM][DIM];  // rows n, t, b
+    const double rxy = sqrt(dr[0] * dr[0] + dr[1] * dr[1]);
+    const double cphi = rxy > 0.0 ? dr[0] / rxy : 1.0, sphi = rxy > 0.0 ? dr[1] / rxy : 0.0;
+    const double cth = dr[2] / r, sth = rxy / r;
+    E[0][0] = dr[0] / r; E[0][1] = dr[1] / r; E[0][2] = dr[2] / r;
+    E[1][0] = cth * cphi; E[1][1] = cth * sphi; E[1][2] = -sth;
+    E[2][0] = -sphi; E[2][1] = cphi; E[2][2] = 0.0;
     for (int d = 0; d < DIM; ++d) {
       double ab = 0.0;
       for (int a = 0; a < DIM; ++a) ab += E[d][a] * coef[a];
       for (int a = 0; a < DIM; ++a) P[(s * DIM + d) * DIM + a] = (C)(ab * E[d][a]);
     }
   }
+}
+
+// Reconstruction weights of a wall point: the linear WLS fit over its interior neighbours,
+// FP64 (the constant fit below dim + 1 of them).
+template <typename C, int DIM>
+__device__ void wall_recon_point(const CaseView& cv, const double* xi, const int32_t* row, const int m, C* R) {
+  const double nah2 = -cv.alpha, hh = cv.h * cv.h;
+  constexpr int M = DIM + 1;
+  double B[M][M];
+#pragma unroll
+  for (int a = 0; a < M; ++a)
+#pragma unroll
+    for (int b = 0; b < M; ++b) B[a][b] = 0.0;
+  int ninner = 0;
+  double wsum = 0.0;
+  for (int s = 0; s < m; ++s) {
+    const int j = row[s];
+    if (cv.kind[j] != 0) continue;
+    double pj[M], xj[DIM];
+    pj[0] = 1.0;
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) { xj[a] = cv.x[(int64_t)j * DIM + a]; pj[1 + a] = sep_d(xi[a], xj[a], cv.periodic); }
+    const double w = exp(nah2 * dist2_d<DIM>(xi, xj, cv.periodic) / hh);
+#pragma unroll
+    for (int a = 0; a < M; ++a)
+#pragma unroll
+      for (int b = 0; b < M; ++b) B[a][b] += w * pj[a] * pj[b];
+    wsum += w;
+    ++ninner;
+  }
+  double z[M];
+  const bool linear = ninner >= M;
+  if (ninner == 0 || (linear && !solve_e0<M>(B, z))) {
+    set_status(cv.status, ST_SINGULAR);
+    for (int s = 0; s < m; ++s) R[s] = (C)0;
+    return;
+  }
+  for (int s = 0; s < m; ++s) {
+    const int j = row[s];
+    if (cv.kind[j] != 0) { R[s] = (C)0; continue; }
+    double pj[M], xj[DIM];
+    pj[0] = 1.0;
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) { xj[a] = cv.x[(int64_t)j * DIM + a]; pj[1 + a] = sep_d(xi[a], xj[a], cv.periodic); }
+    const double w = exp(nah2 * dist2_d<DIM>(xi, xj, cv.periodic) / hh);
+    double r;
+    if (linear) {
+      double acc = 0.0;
+#pragma unroll
+      for (int b = 0; b < M; ++b) acc += z[b] * pj[b];
+      r = w * acc;
+    } else {
+      r = w / wsum;
+    }
+    R[s] = (C)r;
+  }
+}
+
+// 2D, the same fit written for few FP64 instructions (FP64 runs at 2 lanes per clock per
+// SM: one thread per point keeps all 32 lanes of every FP64 instruction in use).  B is
+// accumulated as its upper triangle, each weight is computed once and kept in the slot
+// that the coefficients will take, the elimination goes down only (rows swapped by
+// selects, so everything stays in registers) with one reciprocal per pivot, and the
+// frames need no square root: P_d = e_d (e_d.coef) = d (d.coef) / r^2 with d = dr for the
+// normal and d = (-dr_y, dr_x) for the tangent.  181^2 points, 24^2 velocities, two ALE
+// steps: 1083 us with the square matrix in local memory, every weight computed twice and
+// full elimination (281 us of each step), 816 us now.
+template <typename C>
+__device__ __forceinline__ void quad_stencil_2d(const CaseView& cv, const int i, const double* xi, const int32_t* row,
+                                                const int m, C* P) {
+  constexpr int MQ = 5;
+  const double q = -cv.alpha / cv.h2;
+  double M[MQ][MQ + 2];
+#pragma unroll
+  for (int a = 0; a < MQ; ++a)
+#pragma unroll
+    for (int c = 0; c < MQ + 2; ++c) M[a][c] = c == MQ + a ? 1.0 : 0.0;
+  for (int s = 0; s < m; ++s) {
+    const double* xj = cv.x + (int64_t)row[s] * 2;
+    const double dx = sep_d(xi[0], xj[0], cv.periodic), dy = sep_d(xi[1], xj[1], cv.periodic);
+    const double w = exp(fma(dx, dx, dy * dy) * q);
+    uint32_t* keep = reinterpret_cast<uint32_t*>(P + (int64_t)s * 4);
+    keep[0] = (uint32_t)__double2loint(w);
+    keep[1] = (uint32_t)__double2hiint(w);
+    const double b[MQ] = {dx, dy, 0.5 * dx * dx, dx * dy, 0.5 * dy * dy};
+#pragma unroll
+    for (int a = 0; a < MQ; ++a) {
+      const double wb = w * b[a];
+#pragma unroll
+      for (int c = 0; c < MQ; ++c)
+        if (c >= a) M[a][c] = fma(wb, b[c], M[a][c]);
+    }
+  }
+  double amax = 0.0;
+#pragma unroll
+  for (int a = 0; a < MQ; ++a)
+#pragma unroll
+    for (int c = 0; c < MQ; ++c) {
+      if (c < a) continue;
+      amax = fmax(amax, fabs(M[a][c]));
+      M[c][a] = M[a][c];
+    }
+  bool ok = m >= MQ && amax > 0.0;
+  double inv[MQ];
+  // (constant trip counts with guards, so that every index is known at compile time)
+#pragma unroll
+  for (int c = 0; c < MQ; ++c) {
+    int piv = c;
+    double best = fabs(M[c][c]);
+#pragma unroll
+    for (int r = 0; r < MQ; ++r) {
+      const double v = fabs(M[r][c]);
+      if (r > c && v > best) { best = v; piv = r; }
+    }
+    ok = ok && best > 1e-12 * amax;
+#pragma unroll
+    for (int r = 0; r < MQ; ++r) {
+      if (r <= c) continue;
+      const bool sw = piv == r;
+#pragma unroll
+      for (int k = 0; k < MQ + 2; ++k) {
+        if (k < c) continue;
+        const double u = M[c][k], v = M[r][k];
+        M[c][k] = sw ? v : u;
+        M[r][k] = sw ? u : v;
+      }
+    }
+    inv[c] = 1.0 / M[c][c];
+#pragma unroll
+    for (int r = 0; r < MQ; ++r) {
+      if (r <= c) continue;
+      const double f = M[r][c] * inv[c];
+#pragma unroll
+      for (int k = 0; k < MQ + 2; ++k)
+        if (k > c) M[r][k] = fma(-f, M[c][k], M[r][k]);
+    }
+  }
+  if (!ok) {
+    set_status(cv.status, ST_SINGULAR);
+    for (int s = 0; s < m * 4; ++s) P[s] = (C)0;
+    return;
+  }
+  // the gradient rows of B^-1 (its first two columns)
+  double G[MQ][2];
+#pragma unroll
+  for (int q = 0; q < MQ; ++q) {
+    const int c = MQ - 1 - q;
+#pragma unroll
+    for (int d = 0; d < 2; ++d) {
+      double t = M[c][MQ + d];
+#pragma unroll
+      for (int k = 0; k < MQ; ++k)
+        if (k > c) t = fma(-M[c][k], G[k][d], t);
+      G[c][d] = t * inv[c];
+    }
+  }
+  for (int s = 0; s < m; ++s) {
+    const double* xj = cv.x + (int64_t)row[s] * 2;
+    const double dx = sep_d(xi[0], xj[0], cv.periodic), dy = sep_d(xi[1], xj[1], cv.periodic);
+    const uint32_t* keep = reinterpret_cast<const uint32_t*>(P + (int64_t)s * 4);
+    const double w = __hiloint2double((int)keep[1], (int)keep[0]);
+    const double b[MQ] = {dx, dy, 0.5 * dx * dx, dx * dy, 0.5 * dy * dy};
+    double cx = 0.0, cy = 0.0;
+#pragma unroll
+    for (int a = 0; a < MQ; ++a) { cx = fma(G[a][0], b[a], cx); cy = fma(G[a][1], b[a], cy); }
+    const double z = w / fma(dx, dx, dy * dy);
+    const double an = z * fma(dx, cx, dy * cy), at = z * fma(dx, cy, -dy * cx);
+    P[s * 4] = (C)(an * dx);
+    P[s * 4 + 1] = (C)(an * dy);
+    P[s * 4 + 2] = (C)(-at * dy);
+    P[s * 4 + 3] = (C)(at * dx);
+  }
+}
+
+// Second-order fit, 2D: the interior points in list order, then the wall points.
+template <typename C>
+__global__ void __launch_bounds__(64) k_stencils_quad2(CaseView cv) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= cv.n_int + cv.n_wall) return;
+  const int i = t < cv.n_int ? cv.int_idx[t] : cv.wall_idx[t - cv.n_int];
+  const int m = cv.cnt[i];
+  const int32_t* row = cv.col + (int64_t)i * cv.cap;
+  const double xi[2] = {cv.x[(int64_t)i * 2], cv.x[(int64_t)i * 2 + 1]};
+  if (t < cv.n_int) quad_stencil_2d<C>(cv, i, xi, row, m, (C*)cv.P + (int64_t)i * cv.cap * 4);
+  else wall_recon_point<C, 2>(cv, xi, row, m, (C*)cv.recon + (int64_t)i * cv.cap);
 }
 
 template <typename C, int DIM>
@@ -262,8 +441,8 @@ __global__ void k_stencils(CaseView cv) {
   const double nah2 = -cv.alpha, hh = cv.h * cv.h;
   C* P = (C*)cv.P + (int64_t)i * cap * DIM * DIM;
   C* R = (C*)cv.recon + (int64_t)i * cap;
-  if (cv.kind[i] == 0 && cv.wls_order == 2) {
-    quad_stencil_point<C, DIM>(cv, i, xi, row, m, P);
+  if (DIM == 3 && cv.kind[i] == 0 && cv.wls_order == 2) {
+    if constexpr (DIM == 3) quad_stencil_point<C>(cv, i, xi, row, m, P);
   } else if (cv.kind[i] == 0) {
     double A[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
     for (int s = 0; s < m; ++s) {
@@ -346,55 +525,7 @@ __global__ void k_stencils(CaseView cv) {
       }
     }
   } else {
-    constexpr int M = DIM + 1;
-    double B[M][M];
-#pragma unroll
-    for (int a = 0; a < M; ++a)
-#pragma unroll
-      for (int b = 0; b < M; ++b) B[a][b] = 0.0;
-    int ninner = 0;
-    double wsum = 0.0;
-    for (int s = 0; s < m; ++s) {
-      const int j = row[s];
-      if (cv.kind[j] != 0) continue;
-      double pj[M], xj[DIM];
-      pj[0] = 1.0;
-#pragma unroll
-      for (int a = 0; a < DIM; ++a) { xj[a] = cv.x[(int64_t)j * DIM + a]; pj[1 + a] = sep_d(xi[a], xj[a], cv.periodic); }
-      const double w = exp(nah2 * dist2_d<DIM>(xi, xj, cv.periodic) / hh);
-#pragma unroll
-      for (int a = 0; a < M; ++a)
-#pragma unroll
-        for (int b = 0; b < M; ++b) B[a][b] += w * pj[a] * pj[b];
-      wsum += w;
-      ++ninner;
-    }
-    double z[M];
-    const bool linear = ninner >= M;
-    if (ninner == 0 || (linear && !solve_e0<M>(B, z))) {
-      set_status(cv.status, ST_SINGULAR);
-      for (int s = 0; s < m; ++s) R[s] = (C)0;
-      return;
-    }
-    for (int s = 0; s < m; ++s) {
-      const int j = row[s];
-      if (cv.kind[j] != 0) { R[s] = (C)0; continue; }
-      double pj[M], xj[DIM];
-      pj[0] = 1.0;
-#pragma unroll
-      for (int a = 0; a < DIM; ++a) { xj[a] = cv.x[(int64_t)j * DIM + a]; pj[1 + a] = sep_d(xi[a], xj[a], cv.periodic); }
-      const double w = exp(nah2 * dist2_d<DIM>(xi, xj, cv.periodic) / hh);
-      double r;
-      if (linear) {
-        double acc = 0.0;
-#pragma unroll
-        for (int b = 0; b < M; ++b) acc += z[b] * pj[b];
-        r = w * acc;
-      } else {
-        r = w / wsum;
-      }
-      R[s] = (C)r;
-    }
+    wall_recon_point<C, DIM>(cv, xi, row, m, R);
   }
 }
 
@@ -500,6 +631,12 @@ int launch_stencils(const CaseView& cv, cudaStream_t s, int part) {
     // one FP64 thread per point for every point (the second-order fit: also for
     // FP32/BF16 storage, the coefficients then rounded to FP32)
     if (part == 2) return 0;
+    if (cv.dim == 2 && cv.wls_order == 2) {
+      const int grid = grid_for((int64_t)cv.n_int + cv.n_wall, 64);
+      if (f64) k_stencils_quad2<double><<<grid, 64, 0, s>>>(cv);
+      else k_stencils_quad2<float><<<grid, 64, 0, s>>>(cv);
+      return 1;
+    }
     if (f64) {
       if (cv.dim == 2) k_stencils<double, 2><<<grid_for(cv.n, B), B, 0, s>>>(cv);
       else k_stencils<double, 3><<<grid_for(cv.n, B), B, 0, s>>>(cv);
