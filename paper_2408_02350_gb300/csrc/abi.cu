@@ -120,7 +120,7 @@ struct bgk_ctx {
   CaseView* d_cases[2] = {nullptr, nullptr};
   int2* d_items = nullptr;
   int2* d_witems = nullptr;
-  int n_items = 0, n_witems = 0, capmax = 0, batch_dim = 0, batch_storage = 0;
+  int n_items = 0, n_witems = 0, capmax = 0, nvpmax = 0, batch_dim = 0, batch_storage = 0;
   int batch_warps = 8, batch_grid = 0;
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
   cudaStream_t cap_stream = nullptr;
@@ -479,6 +479,7 @@ int prepare_batch(bgk_ctx* ctx, cudaStream_t s) {
       for (int k = 0; k < v.n_int; ++k) items.push_back(make_int2(ci, k));
       for (int k = 0; k < v.n_wall; ++k) witems.push_back(make_int2(ci, k));
       capmax = std::max(capmax, v.cap);
+      ctx->nvpmax = std::max(ctx->nvpmax, v.NVp);
     }
     if ((st = dalloc(ctx, &ctx->d_items, std::max<size_t>(items.size(), 1)))) return st;
     if ((st = dalloc(ctx, &ctx->d_witems, std::max<size_t>(witems.size(), 1)))) return st;
@@ -509,7 +510,7 @@ int launch_batch_step(bgk_ctx* ctx, int parity, cudaStream_t s) {
   ctx->launches += launch_transport_batch(ctx->d_cases[parity], ctx->d_items, ctx->n_items, ctx->batch_dim,
                                           ctx->batch_storage, ctx->capmax, ctx->batch_warps, ctx->batch_grid, s);
   ctx->launches += launch_walls_batch(ctx->d_cases[parity], ctx->d_witems, ctx->n_witems, ctx->batch_dim,
-                                      ctx->batch_storage, ctx->capmax, s);
+                                      ctx->batch_storage, ctx->capmax, ctx->nvpmax, s);
   CKL(ctx);
   return BGK_OK;
 }
@@ -703,6 +704,7 @@ int bgk_init(const bgk_params* p, int32_t n_cases, const int64_t* n_points, cons
     if ((st = dalloc(ctx, &v.wcls, (size_t)v.n_wall * v.NVp))) return bail(st);
     if ((st = dalloc_bytes(ctx, &v.wvn, (size_t)v.n_wall * v.NVp * c.c_bytes))) return bail(st);
     if ((st = dalloc(ctx, &v.winv, v.n_wall))) return bail(st);
+    if ((st = dalloc(ctx, &v.wunit, (size_t)v.n_wall * (dim + 2)))) return bail(st);
     if ((st = dalloc_bytes(ctx, &v.mw, (size_t)3 * v.NVp * c.c_bytes))) return bail(st);
     if (q.body_wall > 0) {
       if ((st = dalloc(ctx, &v.body, 1))) return bail(st);

@@ -85,6 +85,7 @@ struct CaseView {
   int8_t* wcls;    // [n_wall][NVp] 1 leaving (c_n > 0), 0 arriving
   void* wvn;       // [n_wall][NVp] |c_n|, compute type
   double* winv;    // [n_wall] 1 / sum_{c_n>0} c_n M_w(v)
+  double* wunit;   // [n_wall][dim + 2] moment sums of M_w over the leaving velocities (c_n > 0)
   void* mw;        // [3][NVp] wall Maxwellian G1 (or M) with rho = 1: [0] at rest, [1] lid, [2] body
 
   void* f_in;    // [n][ncomp][NVp] storage type
@@ -193,7 +194,7 @@ int launch_walls(const CaseView& cv, cudaStream_t s);
 int launch_transport_batch(const CaseView* d_cases, const int2* items, int n_items, int dim, int storage, int capmax,
                            int warps, int grid, cudaStream_t s);
 int launch_walls_batch(const CaseView* d_cases, const int2* witems, int n_witems, int dim, int storage, int capmax,
-                       cudaStream_t s);
+                       int nvpmax, cudaStream_t s);
 int launch_move(const CaseView& cv, cudaStream_t s);
 int launch_set_maxwellian(const CaseView& cv, double rho0, const double* u0, double T0, cudaStream_t s);
 int launch_moments(const CaseView& cv, const void* f, cudaStream_t s);

@@ -397,8 +397,8 @@ int launch_transport(const CaseView& cv, cudaStream_t s) {
 // ---------------------------------------------------------------------------
 // walls
 // ---------------------------------------------------------------------------
-// The per-wall-point body (one CTA), shared by the single-case and batched kernels.
-// PH = 0: the whole step.  The sharded step splits it around the sum over all slabs:
+// The wall step of the sharded step (one CTA per wall point), split around the sum over all
+// slabs (the whole step: walls_point_v4):
 // PH = 1 writes the arriving half and the wall sums of the slab to cv.xs[w][2 dim + 6]
 //   [0] sum_{arriving} |c_n| g   [1] sum_{leaving} c_n M_w   [2, dim + 4) moment sums of
 //   the arriving half   [dim + 4, 2 dim + 6) moment sums of M_w over the leaving half;
@@ -406,7 +406,7 @@ int launch_transport(const CaseView& cv, cudaStream_t s) {
 template <int DIM>
 __host__ __device__ constexpr int wall_sums() { return 2 * DIM + 6; }
 
-template <typename S, typename C, int DIM, int PH = 0>
+template <typename S, typename C, int DIM, int PH>
 __device__ __forceinline__ void walls_point(const CaseView& cv, const int w, unsigned char* smem) {
   constexpr int NC = DIM == 2 ? 2 : 1;
   double* s_red = reinterpret_cast<double*>(smem);
@@ -415,8 +415,8 @@ __device__ __forceinline__ void walls_point(const CaseView& cv, const int w, uns
   C* s_r = reinterpret_cast<C*>(smem + RED_BYTES + NODE_BYTES + align16(sizeof(int32_t) * (cv.cap + 1)));
   const int b = cv.wall_idx[w];
   const int nv = cv.nv, NV = cv.NV, NVp = cv.NVp;
-  const int vk0 = PH ? cv.vk0 : 0;
-  if (PH != 2 && threadIdx.x < 32) {
+  const int vk0 = cv.vk0;
+  if (PH == 1 && threadIdx.x < 32) {
     // warp 0 stages the interior neighbours in list order (ballot compaction)
     const int lane = threadIdx.x, m = checked_count(cv.cnt[b], cv.cap, cv.status);
     const int32_t* col = cv.col + (int64_t)b * cv.cap;
@@ -438,7 +438,7 @@ __device__ __forceinline__ void walls_point(const CaseView& cv, const int w, uns
   }
   for (int t = threadIdx.x; t < nv; t += blockDim.x) s_v[t] = (C)cv.vnodes[t];
   __syncthreads();
-  const int mi = PH != 2 ? s_j[0] : 0;
+  const int mi = PH == 1 ? s_j[0] : 0;
   const int64_t rowlen = (int64_t)NC * NVp;
   S* f = reinterpret_cast<S*>(cv.f_out);
   S* fb = f + (int64_t)b * rowlen;
@@ -449,14 +449,14 @@ __device__ __forceinline__ void walls_point(const CaseView& cv, const int w, uns
   const C* Mw = reinterpret_cast<const C*>(cv.mw) + (int64_t)mrow * NVp;
   const C cT = (C)cv.wall_T;
 
-  // flux[0]: sum |c_n| g over the arriving half; flux[1] (PH 1): sum c_n M_w over the
-  // leaving half; part: moment sums of the arriving half (PH 0: of the whole row);
-  // unit (PH 1): moment sums of M_w over the leaving half
+  // (PH 1) flux[0]: sum |c_n| g over the arriving half; flux[1]: sum c_n M_w over the
+  // leaving half; part: moment sums of the arriving half; unit: those of M_w over the
+  // leaving half
   C flux[2] = {(C)0, (C)0};
   C part[DIM + 2], unit[DIM + 2];
 #pragma unroll
   for (int t = 0; t < DIM + 2; ++t) { part[t] = (C)0; unit[t] = (C)0; }
-  if (PH != 2) {
+  if (PH == 1) {
     for (int k = threadIdx.x; k < NV; k += blockDim.x) {
       if (cls[k] == 0) {
         C g[NC];
@@ -483,7 +483,7 @@ __device__ __forceinline__ void walls_point(const CaseView& cv, const int w, uns
         }
         part[DIM + 1] += v2 * g[0];
         if (NC == 2) part[DIM + 1] += g[NC - 1];
-      } else if (PH == 1) {
+      } else {
         const C m0 = Mw[k];
         flux[1] += vn[k] * m0;
         int kk = k + vk0;
@@ -519,46 +519,19 @@ __device__ __forceinline__ void walls_point(const CaseView& cv, const int w, uns
     }
     return;
   }
-  double rho_w;
-  if constexpr (PH == 2) {
-    const double* xw = cv.xs + (int64_t)w * wall_sums<DIM>();
-    rho_w = xw[0] / xw[1];
-  } else {
-    double ftot[1];
-    const C f1[1] = {flux[0]};
-    block_sum0<1, C>(f1, ftot, s_red);
-    rho_w = ftot[0] * cv.winv[w];
-  }
+  const double* xw = cv.xs + (int64_t)w * wall_sums<DIM>();
+  const double rho_w = xw[0] / xw[1];
   const C crw = (C)rho_w;
   for (int k = threadIdx.x; k < NV; k += blockDim.x) {
     if (cls[k] != 0) {
       const C g0 = crw * Mw[k];
       st1(fb + k, g0);
       if (NC == 2) st1(fb + NVp + k, cT * g0);
-      if (PH == 0) {
-        int kk = k;
-        C v2 = (C)0;
-        part[0] += g0;
-#pragma unroll
-        for (int a = 0; a < DIM; ++a) {
-          const C va = s_v[kk % nv];
-          kk /= nv;
-          part[1 + a] += va * g0;
-          v2 += va * va;
-        }
-        part[DIM + 1] += v2 * g0;
-        if (NC == 2) part[DIM + 1] += cT * g0;
-      }
     }
   }
   double tot[DIM + 2];
-  if constexpr (PH == 2) {
-    const double* xw = cv.xs + (int64_t)w * wall_sums<DIM>();
 #pragma unroll
-    for (int q = 0; q < DIM + 2; ++q) tot[q] = xw[2 + q] + rho_w * xw[DIM + 4 + q];
-  } else {
-    block_sum0<DIM + 2, C>(part, tot, s_red);
-  }
+  for (int q = 0; q < DIM + 2; ++q) tot[q] = xw[2 + q] + rho_w * xw[DIM + 4 + q];
   if (threadIdx.x == 0) {
     double rho, Un[3] = {0, 0, 0}, T;
     const double wv = cv.wv;
@@ -569,162 +542,228 @@ __device__ __forceinline__ void walls_point(const CaseView& cv, const int w, uns
   }
 }
 
-// FP32/BF16 storage, the whole wall step (PH = 0 of walls_point): each thread takes 4
-// consecutive velocities, so a neighbour row costs one 16-byte (8-byte for BF16) load
-// per channel instead of four; the leaving half of the loaded values is unused.  The
-// arithmetic per velocity is that of walls_point, with FP32 block sums finished in FP64.
-template <typename S, int DIM>
+// The whole wall step of one wall point by one CTA, 4 consecutive velocities per thread and
+// access.  Bound by latency (a wall point reads about 8 rows, and a cavity has one wall
+// point per lattice point of its boundary), so the chain of dependent steps is short:
+//   - warp 0 compacts the neighbours with a non-zero weight (wall neighbours have weight
+//     zero), so the kinds of the neighbours are not read;
+//   - one reduction: the arriving flux and the arriving half's moment sums together; the
+//     leaving half's moments are rho_w times the sums of M_w tabulated per wall point
+//     (wunit), so they need no second reduction;
+//   - velocity indices split by one float quotient per 4 velocities where a grid row holds
+//     them (ROW), without integer divisions.
+// 160 wall points x 256 velocities (41^2 cavity) 11.6 us with two reductions and a scalar
+// velocity per thread (2D; FP64 15.5 us), 7464 wall points of 24 cavities 123 us.
+// Threads from wall_threads(NVp) on only take part in the barriers, so a wider launch
+// (the batched one) computes the same bits.
+__host__ __device__ inline int wall_threads(int NVp) {
+  const int t = (NVp / 4 + 31) / 32 * 32;
+  return t < 256 ? t : 256;
+}
+
+template <typename C> struct WallNodes;
+template <> struct WallNodes<float> {
+  static __device__ __forceinline__ const float* of(const CaseView& cv) { return cv.vnodes_f; }
+};
+template <> struct WallNodes<double> {
+  static __device__ __forceinline__ const double* of(const CaseView& cv) { return cv.vnodes; }
+};
+
+// Shared memory of the body: neighbours and weights [cap], nodes [64], sums [8 warps][8],
+// rho_w, the neighbour count.
+__host__ __device__ inline size_t wall_smem(int cap) {
+  return align16(sizeof(double) * (size_t)cap) + align16(sizeof(int32_t) * cap) + 64 * 8 + 64 * 8 + 16;
+}
+
+template <typename S, typename C, int DIM>
 __device__ __forceinline__ void walls_point_v4(const CaseView& cv, const int w, unsigned char* smem) {
-  constexpr int NC = DIM == 2 ? 2 : 1;
-  double* s_red = reinterpret_cast<double*>(smem);
-  float* s_v = reinterpret_cast<float*>(smem + RED_BYTES);
-  int32_t* s_j = reinterpret_cast<int32_t*>(smem + RED_BYTES + NODE_BYTES);
-  float* s_r = reinterpret_cast<float*>(smem + RED_BYTES + NODE_BYTES + align16(sizeof(int32_t) * (cv.cap + 1)));
+  constexpr int NC = DIM == 2 ? 2 : 1, NS = DIM + 3;
+  const int cap = cv.cap;
+  C* s_r = reinterpret_cast<C*>(smem);
+  unsigned char* q0 = smem + align16(sizeof(double) * (size_t)cap);
+  int32_t* s_j = reinterpret_cast<int32_t*>(q0);
+  q0 += align16(sizeof(int32_t) * cap);
+  C* s_v = reinterpret_cast<C*>(q0);
+  C* s_sum = reinterpret_cast<C*>(q0 + 512);
+  double* s_rho = reinterpret_cast<double*>(q0 + 1024);
+  int32_t* s_mi = reinterpret_cast<int32_t*>(q0 + 1032);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b = cv.wall_idx[w];
-  const int nv = cv.nv, NV = cv.NV, NVp = cv.NVp;
-  if (threadIdx.x < 32) {
-    const int lane = threadIdx.x, m = checked_count(cv.cnt[b], cv.cap, cv.status);
-    const int32_t* col = cv.col + (int64_t)b * cv.cap;
-    const float* R = reinterpret_cast<const float*>(cv.recon) + (int64_t)b * cv.cap;
+  const int nv = cv.nv, NV = cv.NV, NVp = cv.NVp, nchunk = NVp >> 2;
+  const int T = wall_threads(NVp);
+  if (tid < 32) {
+    const int m = checked_count(cv.cnt[b], cap, cv.status);
+    const int32_t* col = cv.col + (int64_t)b * cap;
+    const C* R = reinterpret_cast<const C*>(cv.recon) + (int64_t)b * cap;
     int mi = 0;
     for (int s0 = 0; s0 < m; s0 += 32) {
       const int s = s0 + lane;
       const int j = s < m ? checked_index(col[s], cv.n, b, cv.status) : 0;
-      const bool in = s < m && cv.kind[j] == 0;
-      const unsigned bal = __ballot_sync(0xffffffffu, in);
-      if (in) {
+      const C r = s < m ? R[s] : (C)0;
+      const unsigned bal = __ballot_sync(0xffffffffu, r != (C)0);
+      if (r != (C)0) {
         const int pos = mi + __popc(bal & ((1u << lane) - 1u));
-        s_j[1 + pos] = j;
-        s_r[pos] = R[s];
+        s_j[pos] = j;
+        s_r[pos] = r;
       }
       mi += __popc(bal);
     }
-    if (lane == 0) s_j[0] = mi;
+    if (lane == 0) *s_mi = mi;
   }
-  for (int t = threadIdx.x; t < nv; t += blockDim.x) s_v[t] = cv.vnodes_f[t];
+  for (int t = tid; t < nv; t += blockDim.x) s_v[t] = WallNodes<C>::of(cv)[t];
   __syncthreads();
-  const int mi = s_j[0];
+  const int mi = *s_mi;
   const int64_t rowlen = (int64_t)NC * NVp;
   S* f = reinterpret_cast<S*>(cv.f_out);
   S* fb = f + (int64_t)b * rowlen;
   const int8_t* cls = cv.wcls + (int64_t)w * NVp;
-  const float* vn = reinterpret_cast<const float*>(cv.wvn) + (int64_t)w * NVp;
-  const int kb = cv.kind[b];
-  const int mrow = kb == cv.lid_wall ? 1 : (cv.body_wall > 0 && kb == cv.body_wall ? 2 : 0);
-  const float* Mw = reinterpret_cast<const float*>(cv.mw) + (int64_t)mrow * NVp;
-  const float cT = (float)cv.wall_T;
-  const int nchunk = NVp >> 2;
+  const C* vn = reinterpret_cast<const C*>(cv.wvn) + (int64_t)w * NVp;
+  const float inv_nv = 1.0f / (float)nv;
+  const bool row = nv % 4 == 0;
 
-  float flux[1] = {0.0f};
-  float part[DIM + 2];
+  // sums over the arriving half: flux, sum g, sum v g, sum |v|^2 g (+ sum h)
+  C sum[NS];
 #pragma unroll
-  for (int t = 0; t < DIM + 2; ++t) part[t] = 0.0f;
-  for (int ch = threadIdx.x; ch < nchunk; ch += blockDim.x) {
+  for (int t = 0; t < NS; ++t) sum[t] = (C)0;
+  for (int ch = tid; ch < nchunk; ch += T) {
+    if (tid >= T) break;
     const int k0 = 4 * ch;
     const char4 c4 = *reinterpret_cast<const char4*>(cls + k0);
     const bool arr[4] = {c4.x == 0 && k0 < NV, c4.y == 0 && k0 + 1 < NV, c4.z == 0 && k0 + 2 < NV,
                          c4.w == 0 && k0 + 3 < NV};
     if (!(arr[0] || arr[1] || arr[2] || arr[3])) continue;
-    float g[NC][4];
+    C g[NC][4];
 #pragma unroll
     for (int c = 0; c < NC; ++c)
 #pragma unroll
-      for (int e = 0; e < 4; ++e) g[c][e] = 0.0f;
+      for (int e = 0; e < 4; ++e) g[c][e] = (C)0;
+#pragma unroll 4
     for (int s = 0; s < mi; ++s) {
-      const S* fj = f + (int64_t)s_j[1 + s] * rowlen + k0;
-      const float r = s_r[s];
+      const S* fj = f + (int64_t)s_j[s] * rowlen + k0;
+      const C r = s_r[s];
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
-        float v[4];
+        C v[4];
         ld4(fj + (int64_t)c * NVp, v);
 #pragma unroll
         for (int e = 0; e < 4; ++e) g[c][e] += r * v[e];
       }
     }
-    const float4 vn4 = *reinterpret_cast<const float4*>(vn + k0);
-    const float vnv[4] = {vn4.x, vn4.y, vn4.z, vn4.w};
+    C vnv[4];
+    ld4(vn + k0, vnv);
+    int ia[4][DIM];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      if (row && e > 0) {
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) ia[e][a] = ia[0][a] + (a == 0 ? e : 0);
+      } else {
+        int kk = k0 + e < NV ? k0 + e : 0;
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) {
+          const int q = fdiv_small(kk, inv_nv);
+          ia[e][a] = kk - q * nv;
+          kk = q;
+        }
+      }
+    }
+    if (arr[0] && arr[1] && arr[2] && arr[3]) {
+#pragma unroll
+      for (int c = 0; c < NC; ++c) st4(fb + (int64_t)c * NVp + k0, g[c]);
+    }
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
       if (!arr[e]) continue;
+      if (!(arr[0] && arr[1] && arr[2] && arr[3])) {
 #pragma unroll
-      for (int c = 0; c < NC; ++c) st1(fb + (int64_t)c * NVp + k0 + e, g[c][e]);
-      flux[0] += vnv[e] * g[0][e];
-      int kk = k0 + e;
-      float v2 = 0.0f;
-      part[0] += g[0][e];
+        for (int c = 0; c < NC; ++c) st1(fb + (int64_t)c * NVp + k0 + e, g[c][e]);
+      }
+      const C g0 = g[0][e];
+      sum[0] += vnv[e] * g0;
+      sum[1] += g0;
+      C v2 = (C)0;
 #pragma unroll
       for (int a = 0; a < DIM; ++a) {
-        const float va = s_v[kk % nv];
-        kk /= nv;
-        part[1 + a] += va * g[0][e];
+        const C va = s_v[ia[e][a]];
+        sum[2 + a] += va * g0;
         v2 += va * va;
       }
-      part[DIM + 1] += v2 * g[0][e];
-      if (NC == 2) part[DIM + 1] += g[NC - 1][e];
+      sum[DIM + 2] += v2 * g0;
+      if (NC == 2) sum[DIM + 2] += g[NC - 1][e];
     }
   }
-  double ftot[1];
-  block_sum0<1, float>(flux, ftot, s_red);
-  const double rho_w = ftot[0] * cv.winv[w];
-  const float crw = (float)rho_w;
-  for (int ch = threadIdx.x; ch < nchunk; ch += blockDim.x) {
+#pragma unroll
+  for (int t = 0; t < NS; ++t) {
+    const C x = warp_sum(sum[t]);
+    if (lane == 0) s_sum[warp * 8 + t] = x;
+  }
+  __syncthreads();
+  if (tid < 32) {
+    // lane t: the total of sum t over the warps, in FP64
+    double tot = 0.0;
+    if (lane < NS)
+      for (int q = 0; q < (T >> 5); ++q) tot += (double)s_sum[q * 8 + lane];
+    const double rho_w = __shfl_sync(0xffffffffu, tot, 0) * cv.winv[w];
+    if (lane == 0) *s_rho = rho_w;
+    const double all = lane >= 1 && lane < NS ? fma(rho_w, cv.wunit[(int64_t)w * (DIM + 2) + lane - 1], tot) : 0.0;
+    double m[DIM + 2];
+#pragma unroll
+    for (int q = 0; q < DIM + 2; ++q) m[q] = __shfl_sync(0xffffffffu, all, q + 1);
+    if (lane == 0) {
+      double rho, Un[3] = {0, 0, 0}, Tn;
+      finish_moments<DIM>(m, cv.wv, &rho, Un, &Tn);
+      double* mo = cv.mom + (int64_t)b * MOM_STRIDE;
+      mo[0] = rho; mo[1] = Un[0]; mo[2] = Un[1]; mo[3] = Un[2]; mo[4] = Tn;
+      if (!(rho_w >= 0.0) || !isfinite(rho_w)) set_status(cv.status, ST_NONFINITE);
+    }
+  }
+  __syncthreads();
+  const int kb = cv.kind[b];
+  const int mrow = kb == cv.lid_wall ? 1 : (cv.body_wall > 0 && kb == cv.body_wall ? 2 : 0);
+  const C* Mw = reinterpret_cast<const C*>(cv.mw) + (int64_t)mrow * NVp;
+  const C crw = (C)*s_rho, cT = (C)cv.wall_T;
+  for (int ch = tid; ch < nchunk; ch += T) {
+    if (tid >= T) break;
     const int k0 = 4 * ch;
     const char4 c4 = *reinterpret_cast<const char4*>(cls + k0);
     const bool lv[4] = {c4.x != 0, c4.y != 0, c4.z != 0, c4.w != 0};
     if (!(lv[0] || lv[1] || lv[2] || lv[3])) continue;
-    const float4 m4 = *reinterpret_cast<const float4*>(Mw + k0);
-    const float mw[4] = {m4.x, m4.y, m4.z, m4.w};
+    C g[4], h[4];
+    ld4(Mw + k0, g);
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      if (!lv[e]) continue;
-      const float g0 = crw * mw[e];
-      st1(fb + k0 + e, g0);
-      if (NC == 2) st1(fb + NVp + k0 + e, cT * g0);
-      int kk = k0 + e;
-      float v2 = 0.0f;
-      part[0] += g0;
+    for (int e = 0; e < 4; ++e) { g[e] = crw * g[e]; h[e] = cT * g[e]; }
+    if (lv[0] && lv[1] && lv[2] && lv[3]) {
+      st4(fb + k0, g);
+      if (NC == 2) st4(fb + NVp + k0, h);
+    } else {
 #pragma unroll
-      for (int a = 0; a < DIM; ++a) {
-        const float va = s_v[kk % nv];
-        kk /= nv;
-        part[1 + a] += va * g0;
-        v2 += va * va;
-      }
-      part[DIM + 1] += v2 * g0;
-      if (NC == 2) part[DIM + 1] += cT * g0;
+      for (int e = 0; e < 4; ++e)
+        if (lv[e]) {
+          st1(fb + k0 + e, g[e]);
+          if (NC == 2) st1(fb + NVp + k0 + e, h[e]);
+        }
     }
   }
-  double tot[DIM + 2];
-  block_sum0<DIM + 2, float>(part, tot, s_red);
-  if (threadIdx.x == 0) {
-    double rho, Un[3] = {0, 0, 0}, T;
-    const double wv = cv.wv;
-    finish_moments<DIM>(tot, wv, &rho, Un, &T);
-    double* mo = cv.mom + (int64_t)b * MOM_STRIDE;
-    mo[0] = rho; mo[1] = Un[0]; mo[2] = Un[1]; mo[3] = Un[2]; mo[4] = T;
-    if (!(rho_w >= 0.0) || !isfinite(rho_w)) set_status(cv.status, ST_NONFINITE);
-  }
 }
 
-template <typename S, int DIM>
+template <typename S, typename C, int DIM>
 __global__ void __launch_bounds__(256) k_walls_v4(const CaseView cv) {
   extern __shared__ __align__(16) unsigned char smem[];
-  walls_point_v4<S, DIM>(cv, blockIdx.x, smem);
+  walls_point_v4<S, C, DIM>(cv, blockIdx.x, smem);
 }
 
-template <typename S, typename C, int DIM, int PH = 0>
+template <typename S, typename C, int DIM, int PH>
 __global__ void __launch_bounds__(256) k_walls(const CaseView cv) {
   extern __shared__ __align__(16) unsigned char smem[];
   walls_point<S, C, DIM, PH>(cv, blockIdx.x, smem);
 }
 
-// witems[k] = (case, wall slot): one CTA per wall point of any case (2D: the body of
-// k_walls, so that batched and per-case stepping give the same bits)
+// witems[k] = (case, wall slot): one CTA per wall point of any case
 template <typename S, typename C, int DIM>
 __global__ void __launch_bounds__(256) k_walls_batch(const CaseView* __restrict__ cases, const int2* __restrict__ witems) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int2 e = witems[blockIdx.x];
-  walls_point<S, C, DIM>(cases[e.x], e.y, smem);
+  walls_point_v4<S, C, DIM>(cases[e.x], e.y, smem);
 }
 
 int launch_transport_batch(const CaseView* d_cases, const int2* items, int n_items, int dim, int storage, int capmax,
@@ -750,35 +789,32 @@ int launch_transport_batch(const CaseView* d_cases, const int2* items, int n_ite
 }
 
 int launch_walls_batch(const CaseView* d_cases, const int2* witems, int n_witems, int dim, int storage, int capmax,
-                       cudaStream_t s) {
+                       int nvpmax, cudaStream_t s) {
   if (n_witems == 0) return 0;
-  const size_t smem = RED_BYTES + NODE_BYTES + align16(sizeof(int32_t) * (capmax + 1)) + sizeof(double) * capmax;
+  const size_t smem = wall_smem(capmax);
+  const int threads = wall_threads(nvpmax);
   if (dim == 2) {
-    if (storage == 1) k_walls_batch<float, float, 2><<<n_witems, 256, smem, s>>>(d_cases, witems);
-    else k_walls_batch<__nv_bfloat16, float, 2><<<n_witems, 256, smem, s>>>(d_cases, witems);
+    if (storage == 1) k_walls_batch<float, float, 2><<<n_witems, threads, smem, s>>>(d_cases, witems);
+    else k_walls_batch<__nv_bfloat16, float, 2><<<n_witems, threads, smem, s>>>(d_cases, witems);
   } else {
-    if (storage == 1) k_walls_batch<float, float, 3><<<n_witems, 256, smem, s>>>(d_cases, witems);
-    else k_walls_batch<__nv_bfloat16, float, 3><<<n_witems, 256, smem, s>>>(d_cases, witems);
+    if (storage == 1) k_walls_batch<float, float, 3><<<n_witems, threads, smem, s>>>(d_cases, witems);
+    else k_walls_batch<__nv_bfloat16, float, 3><<<n_witems, threads, smem, s>>>(d_cases, witems);
   }
   return 1;
 }
 
 int launch_walls(const CaseView& cv, cudaStream_t s) {
   if (cv.n_wall == 0) return 0;
-  const int threads = 256;
-  const size_t smem = RED_BYTES + NODE_BYTES + align16(sizeof(int32_t) * (cv.cap + 1)) + sizeof(double) * cv.cap;
-  // 2D keeps the one-velocity-per-thread body: beside the side-chain kernel of an ALE step
-  // the vector body's extra registers (43 against 32) slow the chain more than they save
-  // (201^2 x 32^2 ALE cavity: 0.4925 against 0.4857 ms per step, chain 61 against 53 us);
-  // in 3D, with no side chain, the vector body wins (41^3 x 16^3: 6.45 against 6.63 ms).
+  const int threads = wall_threads(cv.NVp);
+  const size_t smem = wall_smem(cv.cap);
   if (cv.dim == 2) {
-    if (cv.storage == 0) k_walls<double, double, 2><<<cv.n_wall, threads, smem, s>>>(cv);
-    else if (cv.storage == 1) k_walls<float, float, 2><<<cv.n_wall, threads, smem, s>>>(cv);
-    else k_walls<__nv_bfloat16, float, 2><<<cv.n_wall, threads, smem, s>>>(cv);
+    if (cv.storage == 0) k_walls_v4<double, double, 2><<<cv.n_wall, threads, smem, s>>>(cv);
+    else if (cv.storage == 1) k_walls_v4<float, float, 2><<<cv.n_wall, threads, smem, s>>>(cv);
+    else k_walls_v4<__nv_bfloat16, float, 2><<<cv.n_wall, threads, smem, s>>>(cv);
   } else {
-    if (cv.storage == 0) k_walls<double, double, 3><<<cv.n_wall, threads, smem, s>>>(cv);
-    else if (cv.storage == 1) k_walls_v4<float, 3><<<cv.n_wall, threads, smem, s>>>(cv);
-    else k_walls_v4<__nv_bfloat16, 3><<<cv.n_wall, threads, smem, s>>>(cv);
+    if (cv.storage == 0) k_walls_v4<double, double, 3><<<cv.n_wall, threads, smem, s>>>(cv);
+    else if (cv.storage == 1) k_walls_v4<float, float, 3><<<cv.n_wall, threads, smem, s>>>(cv);
+    else k_walls_v4<__nv_bfloat16, float, 3><<<cv.n_wall, threads, smem, s>>>(cv);
   }
   return 1;
 }
@@ -796,8 +832,9 @@ __device__ __forceinline__ const double* wall_velocity(const CaseView& cv, int k
 }
 
 template <typename C, int DIM>
-__global__ void k_wall_tables(CaseView cv) {
-  __shared__ double s_sum[32];
+__global__ void __launch_bounds__(256) k_wall_tables(CaseView cv) {
+  constexpr int NS = DIM + 3;
+  __shared__ double s_sum[8][NS];
   const int w = blockIdx.x;
   const int b = cv.wall_idx[w];
   const int nv = cv.nv, NV = cv.NV, NVp = cv.NVp;
@@ -808,16 +845,20 @@ __global__ void k_wall_tables(CaseView cv) {
   const double* uw = wall_velocity(cv, cv.kind[b], zero);
   const double pi = 3.14159265358979323846, T = cv.wall_T;
   const double pref = DIM == 2 ? 1.0 / (2.0 * pi * T) : 1.0 / pow(2.0 * pi * T, 1.5);
-  double acc = 0.0;
+  // sum_{c_n > 0} c_n M_w, then the moment sums of the stored M_w over those velocities
+  double acc[NS];
+#pragma unroll
+  for (int t = 0; t < NS; ++t) acc[t] = 0.0;
   for (int k = threadIdx.x; k < NVp; k += blockDim.x) {
     int8_t cl = 0;
     double avn = 0.0;
     if (k < NV) {
       int kk = k + cv.vk0;
-      double vn = 0.0, c2 = 0.0;
+      double vn = 0.0, c2 = 0.0, vv[DIM];
 #pragma unroll
       for (int a = 0; a < DIM; ++a) {
         const double va = cv.vnodes[kk % nv];
+        vv[a] = va;
         kk /= nv;
         const double c = __dadd_rn(va, -uw[a]);
         vn = __dadd_rn(vn, __dmul_rn(c, nb[a]));
@@ -825,17 +866,37 @@ __global__ void k_wall_tables(CaseView cv) {
       }
       cl = vn > 0.0 ? 1 : 0;
       avn = fabs(vn);
-      if (cl) acc += vn * (pref * exp(-c2 / (2.0 * T)));
+      if (cl) {
+        const double M = pref * exp(-c2 / (2.0 * T)), m0 = (double)(C)M;
+        acc[0] += vn * M;
+        acc[1] += m0;
+        double v2 = 0.0;
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) {
+          acc[2 + a] += vv[a] * m0;
+          v2 += vv[a] * vv[a];
+        }
+        acc[DIM + 2] += v2 * m0;
+        if (DIM == 2) acc[DIM + 2] += T * m0;
+      }
     }
     cv.wcls[(int64_t)w * NVp + k] = cl;
     reinterpret_cast<C*>(cv.wvn)[(int64_t)w * NVp + k] = (C)avn;
   }
-  acc = warp_sum(acc);
-  if ((threadIdx.x & 31) == 0) s_sum[threadIdx.x >> 5] = acc;
+#pragma unroll
+  for (int t = 0; t < NS; ++t) {
+    const double x = warp_sum(acc[t]);
+    if ((threadIdx.x & 31) == 0) s_sum[threadIdx.x >> 5][t] = x;
+  }
   __syncthreads();
+  if (threadIdx.x >= 1 && threadIdx.x < NS) {
+    double t = 0.0;
+    for (int q = 0; q < (int)(blockDim.x + 31) / 32; ++q) t += s_sum[q][threadIdx.x];
+    cv.wunit[(int64_t)w * (DIM + 2) + threadIdx.x - 1] = t;
+  }
   if (threadIdx.x == 0) {
     double s = 0.0;
-    for (int q = 0; q < (int)(blockDim.x + 31) / 32; ++q) s += s_sum[q];
+    for (int q = 0; q < (int)(blockDim.x + 31) / 32; ++q) s += s_sum[q][0];
     // a velocity slab of a sharded case holds part of this sum (its wall step takes
     // the sum over all slabs instead): no check there
     const bool slab = cv.vk0 != 0 || NV != (DIM == 2 ? nv * nv : nv * nv * nv);
