@@ -75,13 +75,33 @@ __device__ __forceinline__ void block_sum0(const T (&v)[NVAL], double (&out)[NVA
   __syncthreads();
 }
 
-// Shared memory of the warp-per-point kernels with W warps: velocity nodes, lists,
-// stencils, compensated moment sums.
+// Shared memory of the warp-per-point kernels with W warps: per warp the velocity nodes,
+// the list and stencil, and (ks) the compensated moment sums.
 template <int DIM>
-__host__ __device__ inline size_t wp_smem_bytes(int W, int cap) {
-  return 256 * W + align16(sizeof(int32_t) * cap * W) + align16(sizeof(float) * cap * DIM * DIM * W) +
-         sizeof(float) * kahan_floats<DIM>() * W;
+__host__ __device__ inline size_t wp_smem_bytes(int W, int cap, bool ks = true) {
+  return 256 * W + align16(sizeof(float) * list_floats<DIM>(cap) * W) + (ks ? sizeof(float) * kahan_floats<DIM>() * W : 0);
 }
+template <int DIM>
+struct WarpShared {
+  float* v;
+  int32_t* col;
+  float* P;
+  float* k;
+  __device__ __forceinline__ WarpShared(unsigned char* smem, int W, int warp, int cap) {
+    v = reinterpret_cast<float*>(smem) + warp * 64;
+    float* l = reinterpret_cast<float*>(smem + 256 * W);
+    k = reinterpret_cast<float*>(smem + 256 * W + align16(sizeof(float) * list_floats<DIM>(cap) * W)) +
+        warp * kahan_floats<DIM>();
+    if (DIM == 2) {
+      // 16-byte entries of all warps first, then the indices
+      P = l + (size_t)warp * cap * 4;
+      col = reinterpret_cast<int32_t*>(l + (size_t)W * cap * 4) + warp * cap;
+    } else {
+      P = l + (size_t)warp * list_floats<DIM>(cap);
+      col = nullptr;
+    }
+  }
+};
 
 // Warps per CTA of the single-case first-order launch.  The CTA's points are consecutive
 // in Morton order, but a smaller CTA loses less to the uneven neighbour counts of its
@@ -90,22 +110,20 @@ __host__ __device__ inline size_t wp_smem_bytes(int W, int cap) {
 #ifndef BGK_WP_WARPS
 #define BGK_WP_WARPS 4
 #endif
+// Warps per SM: 32 (64 registers); 28 (72 registers) for 2D BF16, whose conversions need
+// them (201^2 x 32^2 ALE: 414 against 432 us per launch; FP32 411 against 406); 16 with 8
+// velocities per lane.
+template <typename S, int DIM, int VPL>
+constexpr int wp_warps_per_sm() { return VPL != 4 ? 16 : (DIM == 2 && sizeof(S) == 2 ? 28 : 32); }
 template <typename S, int DIM, bool ALE, bool ROW, int VPL, bool SH = false, bool AVG = false>
-__global__ void __launch_bounds__(32 * BGK_WP_WARPS, VPL == 4 ? 32 / BGK_WP_WARPS : 16 / BGK_WP_WARPS)
+__global__ void __launch_bounds__(32 * BGK_WP_WARPS, wp_warps_per_sm<S, DIM, VPL>() / BGK_WP_WARPS)
     k_transport_wp(const CaseView cv) {
-  constexpr int DD = DIM * DIM;
   extern __shared__ __align__(16) unsigned char smem[];
   const int W = blockDim.x >> 5, warp = threadIdx.x >> 5;
-  const int cap = cv.cap;
-  float* s_v = reinterpret_cast<float*>(smem) + warp * 64;
-  int32_t* s_col = reinterpret_cast<int32_t*>(smem + 256 * W) + warp * cap;
-  float* s_P0 = reinterpret_cast<float*>(smem + 256 * W + align16(sizeof(int32_t) * cap * W));
-  float* s_P = s_P0 + (size_t)warp * cap * DD;
-  float* s_k = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(s_P0) + align16(sizeof(float) * W * cap * DD)) +
-               warp * kahan_floats<DIM>();
+  const WarpShared<DIM> ws(smem, W, warp, cv.cap);
   const int t = blockIdx.x * W + warp;
   if (t >= cv.n_int) return;
-  transport_point_wp<S, DIM, ALE, ROW, VPL, VPL == 4, SH, AVG>(cv, cv.int_idx[t], s_v, s_col, s_P, s_k);
+  transport_point_wp<S, DIM, ALE, ROW, VPL, VPL == 4, SH, AVG>(cv, cv.int_idx[t], ws.v, ws.col, ws.P, ws.k);
 }
 
 // Staged variant (2D, FP32, nv % 4 == 0): the neighbour rows come through per-warp rings
@@ -121,18 +139,13 @@ __global__ void __launch_bounds__(32 * BGK_WP_WARPS, BGK_STAGE_MINB) k_transport
   extern __shared__ __align__(16) unsigned char smem[];
   const int W = blockDim.x >> 5, warp = threadIdx.x >> 5;
   const int cap = cv.cap;
-  float* s_v = reinterpret_cast<float*>(smem) + warp * 64;
-  int32_t* s_col = reinterpret_cast<int32_t*>(smem + 256 * W) + warp * cap;
-  float* s_P0 = reinterpret_cast<float*>(smem + 256 * W + align16(sizeof(int32_t) * cap * W));
-  float* s_P = s_P0 + (size_t)warp * cap * 4;
-  float* s_k = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(s_P0) + align16(sizeof(float) * W * cap * 4)) +
-               warp * kahan_floats<2>();
+  const WarpShared<2> ws(smem, W, warp, cap);
   unsigned char* ring0 = smem + stage_ring_offset(wp_smem_bytes<2>(W, cap));
   float* s_ring = reinterpret_cast<float*>(ring0 + (size_t)warp * kStageD * kStageG * kStageRowBytes);
   uint64_t* s_bar = reinterpret_cast<uint64_t*>(ring0 + (size_t)W * kStageD * kStageG * kStageRowBytes) + warp * kStageD;
   const int t = blockIdx.x * W + warp;
   if (t >= cv.n_int) return;
-  transport_point_stage<ALE>(cv, cv.int_idx[t], s_v, s_col, s_P, s_k, s_ring, s_bar);
+  transport_point_stage<ALE>(cv, cv.int_idx[t], ws.v, ws.col, ws.P, ws.k, s_ring, s_bar);
 }
 
 // Second-order step, FP32/BF16 storage: one warp per interior point relaxes its output
@@ -205,30 +218,20 @@ __global__ void __launch_bounds__(256) k_shard_relax_wp(const CaseView cv) {
 }
 
 // Fixed points with a mirror-symmetric velocity grid (nv % 4 == 0, NV % 8 == 0): one
-// warp per interior point, each lane a velocity chunk and its mirror chunk; 79
-// registers, 24 warps per SM.  Used in 3D, where it saves a quarter of the
-// per-neighbour instructions (41^3 x 16^3 cavity: 6.63 against 7.50 ms per step with
-// the 8-velocity kernel); in 2D the extra registers cost more than the saved
-// instructions (201^2 x 32^2 fixed points: 0.483 ms at 4 CTAs per SM with spills,
-// 0.561 ms at 3, against 0.447 ms), so 2D keeps the plain kernel.
-#ifndef BGK_MIRROR_MIN_BLOCKS
-#define BGK_MIRROR_MIN_BLOCKS 3
-#endif
+// warp per interior point, each lane a velocity chunk and its mirror chunk; 128 registers,
+// 16 warps per SM, five neighbours' rows in flight per warp (24 warps with 80 registers and
+// two or three neighbours: 5.36 / 5.33 against 4.96 ms, 41^3 x 16^3).  Used in 3D, where it
+// saves a quarter of the per-neighbour instructions; in 2D the extra registers cost more
+// than the saved instructions (201^2 x 32^2 fixed points: 0.483 ms at 4 CTAs per SM with
+// spills, 0.561 ms at 3, against 0.447 ms), so 2D keeps the plain kernel.
 template <typename S, int DIM, bool KS>
-__global__ void __launch_bounds__(256, BGK_MIRROR_MIN_BLOCKS) k_transport_mirror(const CaseView cv) {
-  constexpr int DD = DIM * DIM;
+__global__ void __launch_bounds__(256, 2) k_transport_mirror(const CaseView cv) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int W = blockDim.x >> 5, warp = threadIdx.x >> 5;
-  const int cap = cv.cap;
-  float* s_v = reinterpret_cast<float*>(smem) + warp * 64;
-  int32_t* s_col = reinterpret_cast<int32_t*>(smem + 256 * W) + warp * cap;
-  float* s_P0 = reinterpret_cast<float*>(smem + 256 * W + align16(sizeof(int32_t) * cap * W));
-  float* s_P = s_P0 + (size_t)warp * cap * DD;
-  float* s_k = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(s_P0) + align16(sizeof(float) * W * cap * DD)) +
-               warp * kahan_floats<DIM>();
+  const WarpShared<DIM> ws(smem, W, warp, cv.cap);
   const int t = blockIdx.x * W + warp;
   if (t >= cv.n_int) return;
-  transport_point_mirror<S, DIM, KS>(cv, cv.int_idx[t], s_v, s_col, s_P, s_k);
+  transport_point_mirror<S, DIM, KS>(cv, cv.int_idx[t], ws.v, ws.col, ws.P, ws.k);
 }
 
 // Many cases in one persistent launch: items[k] = (case, interior slot), tiles of W
@@ -247,15 +250,9 @@ __global__ void __launch_bounds__(256, BGK_MIRROR_MIN_BLOCKS) k_transport_mirror
 template <typename S, int DIM>
 __global__ void __launch_bounds__(256, BGK_BATCH_MIN_BLOCKS) k_transport_batch(const CaseView* __restrict__ cases, const int2* __restrict__ items,
                                                              int n_items, int capmax) {
-  constexpr int DD = DIM * DIM;
   extern __shared__ __align__(16) unsigned char smem[];
   const int W = blockDim.x >> 5, warp = threadIdx.x >> 5;
-  float* s_v = reinterpret_cast<float*>(smem) + warp * 64;
-  int32_t* s_col = reinterpret_cast<int32_t*>(smem + 256 * W) + warp * capmax;
-  float* s_P0 = reinterpret_cast<float*>(smem + 256 * W + align16(sizeof(int32_t) * capmax * W));
-  float* s_P = s_P0 + (size_t)warp * capmax * DD;
-  float* s_k = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(s_P0) + align16(sizeof(float) * W * capmax * DD)) +
-               warp * kahan_floats<DIM>();
+  const WarpShared<DIM> ws(smem, W, warp, capmax);
   for (int tile = blockIdx.x; tile * W < n_items; tile += gridDim.x) {
     const int it = tile * W + warp;
     if (it >= n_items) continue;
@@ -263,8 +260,8 @@ __global__ void __launch_bounds__(256, BGK_BATCH_MIN_BLOCKS) k_transport_batch(c
     const CaseView& cv = cases[e.x];
     const int i = cv.int_idx[e.y];
     // (batched stepping takes fixed points only: c = v)
-    if (cv.nv % 4 == 0) transport_point_wp<S, DIM, false, true, 4, BGK_BATCH_KS>(cv, i, s_v, s_col, s_P, s_k);
-    else transport_point_wp<S, DIM, false, false, 4, BGK_BATCH_KS>(cv, i, s_v, s_col, s_P, s_k);
+    if (cv.nv % 4 == 0) transport_point_wp<S, DIM, false, true, 4, BGK_BATCH_KS>(cv, i, ws.v, ws.col, ws.P, ws.k);
+    else transport_point_wp<S, DIM, false, false, 4, BGK_BATCH_KS>(cv, i, ws.v, ws.col, ws.P, ws.k);
     __syncwarp();
   }
 }
@@ -284,8 +281,9 @@ static void launch_transport_wp(const CaseView& cv, cudaStream_t s) {
   if constexpr (DIM == 3) {
     if (BGK_TRANSPORT_MIRROR && !cv.ale && row4 && cv.NV % 8 == 0) {
       auto k = k_transport_mirror<S, DIM, false>;
-      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      k<<<grid, threads, smem, s>>>(cv);
+      const size_t msm = wp_smem_bytes<DIM>(W, cv.cap, false);
+      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)msm);
+      k<<<grid, threads, msm, s>>>(cv);
       return;
     }
   }

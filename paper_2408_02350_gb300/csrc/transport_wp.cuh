@@ -8,11 +8,18 @@
 
 namespace bgk {
 
-// Neighbour rows whose loads the compiler may overlap (unroll of the neighbour loop).
-#ifndef BGK_NBR_UNROLL
-#define BGK_NBR_UNROLL 2
-#endif
-constexpr int kNbrUnroll = BGK_NBR_UNROLL;
+// Neighbour rows whose loads the compiler may overlap (unroll of the neighbour loop), as
+// measured with the row addresses of row_at: the kernels wait for rows that miss L1 (long
+// scoreboard), so more rows in flight pay until the registers cost a CTA per SM.
+//   2D, shared grid row per lane: 4 (201^2 x 32^2 ALE: 1 / 2 / 3 / 4 rows 487 / 410 / 419 /
+//   406 us per launch; BF16 469 / 447 / 445 / 432);
+//   2D, ragged velocity grids: 2 (133^2 x 27^2: 173 us; 1 / 3 / 4 rows 192 / 196 / 190);
+//   3D: 2 (27^3 x 12^3 ALE: 1 / 2 / 3 / 4 rows 944 / 834 / 847 / 834 us);
+//   mirror pairs (two rows per neighbour): 5 at 16 warps per SM (41^3 x 16^3: 2 / 4 / 5 / 6
+//   / 8 neighbours 5.76 / 5.07 / 4.96 / 5.00 / 4.98 ms; 5.33 ms at best with 24 warps).
+template <int DIM, bool ROW>
+__host__ __device__ constexpr int nbr_unroll() { return DIM == 2 && ROW ? 4 : 2; }
+constexpr int kMirrorUnroll = 5;
 
 // ---------------------------------------------------------------------------
 // transport + moments + relaxation, FP32 arithmetic (FP32 or BF16 storage):
@@ -109,6 +116,13 @@ template <typename S, int VPL>
 __device__ __forceinline__ void stv(S* p, const float (&v)[VPL]) {
 #pragma unroll
   for (int q = 0; q < VPL / 4; ++q) st4(p + 4 * q, v + 4 * q);
+}
+
+// Row j of an array whose rows take rb bytes, at the byte address base: one widening
+// 32-bit multiply-add per row (64-bit index arithmetic costs four to eight instructions).
+template <typename S>
+__device__ __forceinline__ const S* row_at(const S* base, const int j, const uint32_t rb) {
+  return reinterpret_cast<const S*>(reinterpret_cast<const char*>(base) + (uint64_t)(uint32_t)j * rb);
 }
 
 // Upwind sums of one neighbour row for the VPL = 2 NP velocities of a lane that lie
@@ -438,6 +452,62 @@ __device__ __forceinline__ void ks_load(const float* s_k, const int lane, float 
   }
 }
 
+// The point's list and stencil in the warp's shared memory.  2D: the indices, then one
+// 16-byte entry per neighbour.  3D: one 48-byte entry per neighbour, rows (P_dx, P_dy,
+// P_dz, .) with the neighbour's index in the first spare word, so that a neighbour costs
+// three 16-byte loads instead of ten 4-byte ones; only the first kList3 neighbours are
+// staged (max_nbrs is sized for dense clouds, 160 for about 80 neighbours, and shared
+// memory for all of it would leave 32 KB of L1 for the neighbour rows); the rest are read
+// from global memory.  With 4-byte entries for all of max_nbrs and 64-bit row indices the
+// 41^3 x 16^3 transport took 5.97 ms per launch (4.96 now), 27^3 x 12^3 ALE 1042 us (834).
+constexpr int kList3 = 96;
+template <int DIM>
+__host__ __device__ constexpr int staged_nbrs(int cap) { return DIM == 3 && cap > kList3 ? kList3 : cap; }
+template <int DIM>
+__host__ __device__ constexpr int list_floats(int cap) { return DIM == 3 ? 12 * staged_nbrs<3>(cap) : 5 * cap; }
+
+template <int DIM>
+__device__ __forceinline__ void stage_list(const CaseView& cv, const int i, const int m, float* s_P, int32_t* s_col) {
+  const int lane = threadIdx.x & 31;
+  const int32_t* col = cv.col + (int64_t)i * cv.cap;
+  const float* P = reinterpret_cast<const float*>(cv.P) + (int64_t)i * cv.cap * DIM * DIM;
+  if constexpr (DIM == 2) {
+    for (int q = lane; q < m; q += 32) s_col[q] = checked_index(col[q], cv.n, i, cv.status);
+    for (int q = lane; q < m * 4; q += 32) s_P[q] = P[q];
+  } else {
+    const int ms = min(m, kList3);
+    for (int q = lane; q < ms; q += 32) s_P[12 * q + 3] = __int_as_float(checked_index(col[q], cv.n, i, cv.status));
+    for (int q = lane; q < ms * 9; q += 32) {
+      const int e = q / 9, r = q - 9 * e;
+      s_P[12 * e + r + r / 3] = P[q];
+    }
+  }
+}
+// Neighbour s (staged): its index, its coefficients into P.
+template <int DIM>
+__device__ __forceinline__ int staged_nbr(const float* s_P, const int32_t* s_col, const int s, float (&P)[DIM * DIM]) {
+  if constexpr (DIM == 2) {
+    const float4 a = reinterpret_cast<const float4*>(s_P)[s];
+    P[0] = a.x; P[1] = a.y; P[2] = a.z; P[3] = a.w;
+    return s_col[s];
+  } else {
+    const float4* e = reinterpret_cast<const float4*>(s_P) + 3 * s;
+    const float4 a = e[0], b = e[1], c = e[2];
+    P[0] = a.x; P[1] = a.y; P[2] = a.z;
+    P[3] = b.x; P[4] = b.y; P[5] = b.z;
+    P[6] = c.x; P[7] = c.y; P[8] = c.z;
+    return __float_as_int(a.w);
+  }
+}
+// Neighbour s from global memory (3D, past the staged ones).
+template <int DIM>
+__device__ __forceinline__ int global_nbr(const CaseView& cv, const int i, const int s, float (&P)[DIM * DIM]) {
+  const float* g = reinterpret_cast<const float*>(cv.P) + ((int64_t)i * cv.cap + s) * DIM * DIM;
+#pragma unroll
+  for (int q = 0; q < DIM * DIM; ++q) P[q] = g[q];
+  return checked_index(cv.col[(int64_t)i * cv.cap + s], cv.n, i, cv.status);
+}
+
 template <typename S, int DIM, bool ALE, bool ROW, int VPL, bool KS, bool SH = false, bool AVG = false>
 __device__ __forceinline__ void transport_point_wp(const CaseView& cv, const int i, float* s_v, int32_t* s_col,
                                                    float* s_P, float* s_k) {
@@ -450,12 +520,8 @@ __device__ __forceinline__ void transport_point_wp(const CaseView& cv, const int
   const float inv_nv = 1.0f / (float)nv;
   const int m = checked_count(cv.cnt[i], cap, cv.status);
   for (int q = lane; q < nv; q += 32) s_v[q] = cv.vnodes_f[q];
-  {
-    const int32_t* col = cv.col + (int64_t)i * cap;
-    const float* P = reinterpret_cast<const float*>(cv.P) + (int64_t)i * cap * DD;
-    for (int q = lane; q < m; q += 32) s_col[q] = checked_index(col[q], cv.n, i, cv.status);
-    for (int q = lane; q < m * DD; q += 32) s_P[q] = P[q];
-  }
+  stage_list<DIM>(cv, i, m, s_P, s_col);
+  const int ms = DIM == 3 ? min(m, kList3) : m;  // staged neighbours
   __syncwarp();
 
   float U[DIM];
@@ -464,6 +530,7 @@ __device__ __forceinline__ void transport_point_wp(const CaseView& cv, const int
 
   const int nchunk = NVp / VPL;
   const int nslice = (nchunk + 31) >> 5;
+  const uint32_t rb = (uint32_t)(NC * NVp * (int)sizeof(S));  // bytes of a row
   const int64_t rowlen = (int64_t)NC * NVp;
   const S* fbase = reinterpret_cast<const S*>(cv.f_in);
   const float two_dt = cv.two_dt_f;
@@ -485,6 +552,7 @@ __device__ __forceinline__ void transport_point_wp(const CaseView& cv, const int
     chunk_velocities<DIM, VPL, ROW>(k0 + vk0, nv, NV + vk0, inv_nv, s_v, vel, kin);
     {
     const S* fj0 = fbase + k0;
+    const S* fj1 = fj0 + NVp;
     if (ROW) {
       // velocity pairs in packed FP32x2 arithmetic; the pairs share (v_y, v_z)
       float2 cx[NP];
@@ -500,17 +568,25 @@ __device__ __forceinline__ void transport_point_wp(const CaseView& cv, const int
 #pragma unroll
         for (int c = 0; c < NC; ++c) ap[c][q] = f2(0.0f, 0.0f);
       }
-#pragma unroll kNbrUnroll
-      for (int s = 0; s < m; ++s) {
-        const int j = s_col[s];
-        float P[DD];
-#pragma unroll
-        for (int q = 0; q < DD; ++q) P[q] = s_P[s * DD + q];
-        const S* fj = fj0 + (int64_t)j * rowlen;
+      auto row = [&](const int j, const float (&P)[DD]) {
         float fv[NC][VPL];
 #pragma unroll
-        for (int c = 0; c < NC; ++c) ldv_ro<S, VPL>(fj + (int64_t)c * NVp, fv[c]);
+        for (int c = 0; c < NC; ++c) ldv_ro<S, VPL>(row_at(c ? fj1 : fj0, j, rb), fv[c]);
         row_upwind<DIM, NC, NP>(cx, crest, P, fv, skp, ap);
+      };
+#pragma unroll (nbr_unroll<DIM, true>())
+      for (int s = 0; s < ms; ++s) {
+        float P[DD];
+        const int j = staged_nbr<DIM>(s_P, s_col, s, P);
+        row(j, P);
+      }
+      if constexpr (DIM == 3) {
+#pragma unroll 1
+        for (int s = ms; s < m; ++s) {
+          float P[DD];
+          const int j = global_nbr<DIM>(cv, i, s, P);
+          row(j, P);
+        }
       }
 #pragma unroll
       for (int q = 0; q < NP; ++q) {
@@ -536,16 +612,14 @@ __device__ __forceinline__ void transport_point_wp(const CaseView& cv, const int
 #pragma unroll
         for (int c = 0; c < NC; ++c) ap[c][q] = f2(0.0f, 0.0f);
       }
-#pragma unroll kNbrUnroll
-      for (int s = 0; s < m; ++s) {
-        const int j = s_col[s];
-        float P[DD];
-#pragma unroll
-        for (int q = 0; q < DD; ++q) P[q] = s_P[s * DD + q];
-        const S* fj = fj0 + (int64_t)j * rowlen;
+      auto row = [&](const int j, const float (&P)[DD]) {
         float fv[NC][VPL];
 #pragma unroll
-        for (int c = 0; c < NC; ++c) ldv_ro<S, VPL>(fj + (int64_t)c * NVp, fv[c]);
+        for (int c = 0; c < NC; ++c) {
+          // (2D: 64-bit indices here; row_at took 190 against 173 us, 133^2 x 27^2)
+          if constexpr (DIM == 2) ldv_ro<S, VPL>(fj0 + (int64_t)j * rowlen + (int64_t)c * NVp, fv[c]);
+          else ldv_ro<S, VPL>(row_at(fj0, j, rb), fv[c]);
+        }
         float2 mk[NP];
 #pragma unroll
         for (int d = 0; d < DIM; ++d) {
@@ -563,6 +637,20 @@ __device__ __forceinline__ void transport_point_wp(const CaseView& cv, const int
           skp[q] = __fadd2_rn(skp[q], mk[q]);
 #pragma unroll
           for (int c = 0; c < NC; ++c) ap[c][q] = __ffma2_rn(mk[q], f2(fv[c][2 * q], fv[c][2 * q + 1]), ap[c][q]);
+        }
+      };
+#pragma unroll (nbr_unroll<DIM, false>())
+      for (int s = 0; s < ms; ++s) {
+        float P[DD];
+        const int j = staged_nbr<DIM>(s_P, s_col, s, P);
+        row(j, P);
+      }
+      if constexpr (DIM == 3) {
+#pragma unroll 1
+        for (int s = ms; s < m; ++s) {
+          float P[DD];
+          const int j = global_nbr<DIM>(cv, i, s, P);
+          row(j, P);
         }
       }
 #pragma unroll
@@ -609,17 +697,13 @@ __device__ __forceinline__ void transport_point_mirror(const CaseView& cv, const
   const float inv_nv = 1.0f / (float)nv;
   const int m = checked_count(cv.cnt[i], cap, cv.status);
   for (int q = lane; q < nv; q += 32) s_v[q] = cv.vnodes_f[q];
-  {
-    const int32_t* col = cv.col + (int64_t)i * cap;
-    const float* P = reinterpret_cast<const float*>(cv.P) + (int64_t)i * cap * DD;
-    for (int q = lane; q < m; q += 32) s_col[q] = checked_index(col[q], cv.n, i, cv.status);
-    for (int q = lane; q < m * DD; q += 32) s_P[q] = P[q];
-  }
+  stage_list<DIM>(cv, i, m, s_P, s_col);
+  const int ms = DIM == 3 ? min(m, kList3) : m;  // staged neighbours
   __syncwarp();
 
   const int nchunk = NV / (2 * VPL);
   const int nslice = (nchunk + 31) >> 5;
-  const int64_t rowlen = (int64_t)NC * NVp;
+  const uint32_t rb = (uint32_t)(NC * NVp * (int)sizeof(S));  // bytes of a row
   const S* fbase = reinterpret_cast<const S*>(cv.f_in);
   const float two_dt = cv.two_dt_f;
   const float2 neg1 = f2(-1.0f, -1.0f);
@@ -654,18 +738,12 @@ __device__ __forceinline__ void transport_point_mirror(const CaseView& cv, const
       }
       const S* fj0 = fbase + k0;
       const S* fm0 = fbase + km;
-#pragma unroll 2
-      for (int s = 0; s < m; ++s) {
-        const int j = s_col[s];
-        float P[DD];
-#pragma unroll
-        for (int q = 0; q < DD; ++q) P[q] = s_P[s * DD + q];
-        const int64_t o = (int64_t)j * rowlen;
+      auto row = [&](const int j, const float (&P)[DD]) {
         float fv[NC][VPL], fw[NC][VPL];
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
-          ldv_ro<S, VPL>(fj0 + o + (int64_t)c * NVp, fv[c]);
-          ldv_ro<S, VPL>(fm0 + o + (int64_t)c * NVp, fw[c]);
+          ldv_ro<S, VPL>(row_at(fj0 + c * NVp, j, rb), fv[c]);
+          ldv_ro<S, VPL>(row_at(fm0 + c * NVp, j, rb), fw[c]);
         }
         float2 mk[NP], ps[NP];
 #pragma unroll
@@ -694,6 +772,20 @@ __device__ __forceinline__ void transport_point_mirror(const CaseView& cv, const
 #pragma unroll
           for (int c = 0; c < NC; ++c)
             aq[c][r] = __ffma2_rn(mr, f2(fw[c][2 * r], fw[c][2 * r + 1]), aq[c][r]);
+        }
+      };
+#pragma unroll kMirrorUnroll
+      for (int s = 0; s < ms; ++s) {
+        float P[DD];
+        const int j = staged_nbr<DIM>(s_P, s_col, s, P);
+        row(j, P);
+      }
+      if constexpr (DIM == 3) {
+#pragma unroll 1
+        for (int s = ms; s < m; ++s) {
+          float P[DD];
+          const int j = global_nbr<DIM>(cv, i, s, P);
+          row(j, P);
         }
       }
 #pragma unroll
