@@ -121,7 +121,8 @@ struct bgk_ctx {
   int2* d_items = nullptr;
   int2* d_witems = nullptr;
   int n_items = 0, n_witems = 0, capmax = 0, nvpmax = 0, batch_dim = 0, batch_storage = 0;
-  int batch_warps = 8, batch_grid = 0;
+  // (4 warps per CTA: 1409 us per step of 24 cavities of up to 121^2 points, 1432 with 8)
+  int batch_warps = 4, batch_grid = 0;
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
   cudaStream_t cap_stream = nullptr;
   cudaStream_t side = nullptr;  // ALE motion and next-step lists, concurrent with the wall kernel

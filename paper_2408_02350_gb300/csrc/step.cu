@@ -110,13 +110,14 @@ struct WarpShared {
 #ifndef BGK_WP_WARPS
 #define BGK_WP_WARPS 4
 #endif
-// Warps per SM: 32 (64 registers); 28 (72 registers) for 2D BF16, whose conversions need
-// them (201^2 x 32^2 ALE: 414 against 432 us per launch; FP32 411 against 406); 16 with 8
-// velocities per lane.
-template <typename S, int DIM, int VPL>
-constexpr int wp_warps_per_sm() { return VPL != 4 ? 16 : (DIM == 2 && sizeof(S) == 2 ? 28 : 32); }
+// Warps per SM: 32 (64 registers); 28 (72 registers) for 2D BF16 with aligned velocity
+// rows, whose conversions need them (201^2 x 32^2 ALE: 414 against 432 us per launch; FP32
+// 411 against 406; ragged BF16, 190^2 x 30^2 ALE, two steps: 1069 against 1051 us); 16 with
+// 8 velocities per lane.
+template <typename S, int DIM, int VPL, bool ROW>
+constexpr int wp_warps_per_sm() { return VPL != 4 ? 16 : (DIM == 2 && ROW && sizeof(S) == 2 ? 28 : 32); }
 template <typename S, int DIM, bool ALE, bool ROW, int VPL, bool SH = false, bool AVG = false>
-__global__ void __launch_bounds__(32 * BGK_WP_WARPS, wp_warps_per_sm<S, DIM, VPL>() / BGK_WP_WARPS)
+__global__ void __launch_bounds__(32 * BGK_WP_WARPS, wp_warps_per_sm<S, DIM, VPL, ROW>() / BGK_WP_WARPS)
     k_transport_wp(const CaseView cv) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int W = blockDim.x >> 5, warp = threadIdx.x >> 5;

@@ -179,13 +179,20 @@ __device__ __forceinline__ void kahan_add(const float (&ps)[N], float (&msum)[N]
   }
 }
 
+// Whether the slice epilogue and the relaxation run in packed FP32x2 pairs when the lane's
+// velocities do not share a grid row: FP32 storage (133^2 x 27^2: 169 against 174 us per
+// launch; a step of 24 cavities, most of them ragged, 1379 against 1409 us).  BF16 keeps
+// one velocity at a time, whose roundings its stored values repeat.
+template <typename S>
+__host__ __device__ constexpr bool packed_ragged() { return sizeof(S) == 4; }
+
 // End of a velocity slice: f~ = f_i - 2 dt (acc - sk f_i) for the lane's VPL
 // velocities, written to the output row (and to the adjoint's tape when one is
 // attached); the slice's moment sums are Kahan-added to the lane's running sums.
 // AVG (second stage of the two-stage transport): f~ = (f_avg,i + f~) / 2, f_avg the
 // state at the start of the step, whose row i is read before the output overwrites it.
 // ROW: the lane's velocities share every component but the first (then the sums of
-// v_a g for a >= 1 are v_a sum g), and f~ is formed in packed FP32x2 pairs.
+// v_a g for a >= 1 are v_a sum g).  Packed FP32x2 pairs with ROW and for FP32 storage.
 template <typename S, int DIM, int NC, int VPL, bool AVG = false, bool ROW = false>
 __device__ __forceinline__ void slice_out(const CaseView& cv, const int i, const int k0, const float (&vel)[VPL][DIM],
                                           const bool (&kin)[VPL], const float (&acc)[NC][VPL],
@@ -204,7 +211,7 @@ __device__ __forceinline__ void slice_out(const CaseView& cv, const int i, const
     for (int c = 0; c < NC; ++c) ldv<S, VPL>(fa + (int64_t)c * NVp + k0, fav[c]);
   }
   float ps[DIM + 2];
-  if constexpr (ROW && VPL % 2 == 0) {
+  if constexpr (ROW || packed_ragged<S>()) {
     constexpr int NP = VPL / 2;
     const float2 ntd = f2(-two_dt, -two_dt);
 #pragma unroll
@@ -225,24 +232,49 @@ __device__ __forceinline__ void slice_out(const CaseView& cv, const int i, const
 #pragma unroll
         for (int c = 0; c < NC; ++c) ft[c][e] = kin[e] ? ft[c][e] : 0.0f;
     }
-    // sum g, sum v_x g, sum |v|^2 g (+ sum h) in pairs; |v|^2 = v_x^2 + r2
-    float r2 = 0.0f;
+    float2 gs = f2(0.0f, 0.0f), wg = gs, hs = gs;
+    if constexpr (ROW) {
+      // sum g, sum v_x g, sum |v|^2 g (+ sum h) in pairs; |v|^2 = v_x^2 + r2
+      float r2 = 0.0f;
 #pragma unroll
-    for (int a = 1; a < DIM; ++a) r2 = fmaf(vel[0][a], vel[0][a], r2);
-    float2 gs = f2(0.0f, 0.0f), xg = gs, wg = gs, hs = gs;
+      for (int a = 1; a < DIM; ++a) r2 = fmaf(vel[0][a], vel[0][a], r2);
+      float2 xg = gs;
 #pragma unroll
-    for (int q = 0; q < NP; ++q) {
-      const float2 g = f2(ft[0][2 * q], ft[0][2 * q + 1]);
-      const float2 vx = f2(vel[2 * q][0], vel[2 * q + 1][0]);
-      gs = __fadd2_rn(gs, g);
-      xg = __ffma2_rn(vx, g, xg);
-      wg = __ffma2_rn(__ffma2_rn(vx, vx, f2(r2, r2)), g, wg);
-      if (NC == 2) hs = __fadd2_rn(hs, f2(ft[NC - 1][2 * q], ft[NC - 1][2 * q + 1]));
+      for (int q = 0; q < NP; ++q) {
+        const float2 g = f2(ft[0][2 * q], ft[0][2 * q + 1]);
+        const float2 vx = f2(vel[2 * q][0], vel[2 * q + 1][0]);
+        gs = __fadd2_rn(gs, g);
+        xg = __ffma2_rn(vx, g, xg);
+        wg = __ffma2_rn(__ffma2_rn(vx, vx, f2(r2, r2)), g, wg);
+        if (NC == 2) hs = __fadd2_rn(hs, f2(ft[NC - 1][2 * q], ft[NC - 1][2 * q + 1]));
+      }
+      ps[0] = gs.x + gs.y;
+      ps[1] = xg.x + xg.y;
+#pragma unroll
+      for (int a = 1; a < DIM; ++a) ps[1 + a] = vel[0][a] * ps[0];
+    } else {
+      // the same with every velocity's own components
+      float2 vg[DIM];
+#pragma unroll
+      for (int a = 0; a < DIM; ++a) vg[a] = gs;
+#pragma unroll
+      for (int q = 0; q < NP; ++q) {
+        const float2 g = f2(ft[0][2 * q], ft[0][2 * q + 1]);
+        gs = __fadd2_rn(gs, g);
+        float2 v2 = f2(0.0f, 0.0f);
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) {
+          const float2 va = f2(vel[2 * q][a], vel[2 * q + 1][a]);
+          vg[a] = __ffma2_rn(va, g, vg[a]);
+          v2 = a == 0 ? __fmul2_rn(va, va) : __ffma2_rn(va, va, v2);
+        }
+        wg = __ffma2_rn(v2, g, wg);
+        if (NC == 2) hs = __fadd2_rn(hs, f2(ft[NC - 1][2 * q], ft[NC - 1][2 * q + 1]));
+      }
+      ps[0] = gs.x + gs.y;
+#pragma unroll
+      for (int a = 0; a < DIM; ++a) ps[1 + a] = vg[a].x + vg[a].y;
     }
-    ps[0] = gs.x + gs.y;
-    ps[1] = xg.x + xg.y;
-#pragma unroll
-    for (int a = 1; a < DIM; ++a) ps[1 + a] = vel[0][a] * ps[0];
     ps[DIM + 1] = NC == 2 ? (wg.x + wg.y) + (hs.x + hs.y) : wg.x + wg.y;
   } else {
 #pragma unroll
@@ -337,19 +369,29 @@ __device__ __forceinline__ void relax_point(const CaseView& cv, const int i, con
     float ft[NC][VPL], out[NC][VPL];
 #pragma unroll
     for (int c = 0; c < NC; ++c) ldv<S, VPL>(fo + (int64_t)c * NVp + k0, ft[c]);
-    if constexpr (ROW && VPL % 2 == 0) {
-      // in packed pairs: |v - U|^2 = (v_x - U_x)^2 + r2, r2 shared by the lane's velocities;
-      // M from 2^(l2 |v - U|^2), l2 = -log2(e) / (2 T)
+    if constexpr (ROW || packed_ragged<S>()) {
+      // in packed pairs: |v - U|^2 (ROW: (v_x - U_x)^2 + r2, r2 shared by the lane's
+      // velocities); M from 2^(l2 |v - U|^2), l2 = -log2(e) / (2 T)
       float r2 = 0.0f;
+      if (ROW) {
 #pragma unroll
-      for (int a = 1; a < DIM; ++a) {
-        const float d = vel[0][a] - Un[a];
-        r2 = fmaf(d, d, r2);
+        for (int a = 1; a < DIM; ++a) {
+          const float d = vel[0][a] - Un[a];
+          r2 = fmaf(d, d, r2);
+        }
       }
 #pragma unroll
       for (int q = 0; q < VPL / 2; ++q) {
+        float2 c2 = f2(r2, r2);
+        if (!ROW) {
+#pragma unroll
+          for (int a = 1; a < DIM; ++a) {
+            const float2 d = __fadd2_rn(f2(vel[2 * q][a], vel[2 * q + 1][a]), f2(-Un[a], -Un[a]));
+            c2 = a == 1 ? __fmul2_rn(d, d) : __ffma2_rn(d, d, c2);
+          }
+        }
         const float2 dx = __fadd2_rn(f2(vel[2 * q][0], vel[2 * q + 1][0]), f2(-Un[0], -Un[0]));
-        const float2 ea = __fmul2_rn(__ffma2_rn(dx, dx, f2(r2, r2)), f2(l2, l2));
+        const float2 ea = __fmul2_rn(__ffma2_rn(dx, dx, c2), f2(l2, l2));
         const float2 bM = __fmul2_rn(f2(pref, pref), f2(exp2_approx(ea.x), exp2_approx(ea.y)));
         const float2 o0 = __ffma2_rn(f2(ca, ca), f2(ft[0][2 * q], ft[0][2 * q + 1]), bM);
         out[0][2 * q] = o0.x; out[0][2 * q + 1] = o0.y;
