@@ -20,6 +20,7 @@
 
 #include "bgk_internal.cuh"
 #include "device_common.cuh"
+#include "transport_wp.cuh"
 
 namespace bgk {
 
@@ -28,13 +29,32 @@ constexpr int RED = 16 * 32;  // doubles of block-reduction scratch (16 values x
 
 inline int grid_for(int64_t n, int b) { return (int)((n + b - 1) / b); }
 
+// Sums of up to 8 values over the block.  Within a warp they are reduced transposed (lanes
+// give away half of their sums at each of the first three steps): 9 FP64 additions per
+// warp instead of 5 per value (FP64 runs at 1/64 of the FP32 rate).
 template <int NVAL>
 __device__ __forceinline__ void block_reduce(double (&v)[NVAL], double* scratch) {
+  static_assert(NVAL <= 8, "at most 8 sums");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+  if constexpr (NVAL == 1) {
+    const double s = warp_sum(v[0]);
+    if (lane == 0) scratch[warp] = s;
+  } else {
+    const bool h16 = (lane & 16) != 0, h8 = (lane & 8) != 0, h4 = (lane & 4) != 0;
+    double a[4], b[2];
 #pragma unroll
-  for (int q = 0; q < NVAL; ++q) {
-    double s = warp_sum(v[q]);
-    if (lane == 0) scratch[q * 32 + warp] = s;
+    for (int q = 0; q < 4; ++q) {
+      const double lo = q < NVAL ? v[q < NVAL ? q : 0] : 0.0, hi = q + 4 < NVAL ? v[q + 4 < NVAL ? q + 4 : 0] : 0.0;
+      a[q] = (h16 ? hi : lo) + __shfl_xor_sync(0xffffffffu, h16 ? lo : hi, 16);
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+      b[q] = (h8 ? a[q + 2] : a[q]) + __shfl_xor_sync(0xffffffffu, h8 ? a[q] : a[q + 2], 8);
+    double s = (h4 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, h4 ? b[0] : b[1], 4);
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    const int q = (h16 ? 4 : 0) + (h8 ? 2 : 0) + (h4 ? 1 : 0);
+    if ((lane & 3) == 0 && q < NVAL) scratch[q * 32 + warp] = s;
   }
   __syncthreads();
   if (threadIdx.x < NVAL) {
@@ -491,38 +511,44 @@ __global__ void __launch_bounds__(256) k_objective(CaseView cv, int nlid, double
 // FP32 path: warp-per-point adjoint kernels (lanes own 4 velocities of each
 // 128-velocity slice, as in the forward transport)
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ int fdiv_small_a(int k, float inv_n) { return (int)(((float)k + 0.5f) * inv_n); }
-
-template <int DIM>
-__device__ __forceinline__ void chunk_vel_a(int k0, int nv, int NV, float inv_nv, const float* s_v, float (&vel)[4][DIM],
-                                            bool (&kin)[4]) {
+// lam_y of the lane's 4 velocities at interior point i: lam1 plus the terms of its wall
+// neighbours (s_wb: point b, wall slot w, slot of i in b).
+template <int NC>
+__device__ __forceinline__ void lam_y4(const CaseView& cv, const float* l1, const float* lam1, const double* wmu,
+                                       const int32_t* s_wb, const int nwb, const int k0, float (&ly)[NC][4]) {
+  const int NVp = cv.NVp;
 #pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    int kk = k0 + e;
-    kin[e] = kk < NV;
-    if (!kin[e]) kk = 0;
+  for (int c = 0; c < NC; ++c) ld4(l1 + (int64_t)c * NVp + k0, ly[c]);
+  for (int q = 0; q < nwb; ++q) {
+    const int b = s_wb[3 * q], w = s_wb[3 * q + 1], slb = s_wb[3 * q + 2];
+    const float r = reinterpret_cast<const float*>(cv.recon)[(int64_t)b * cv.cap + slb];
+    const float mu = (float)wmu[w];
+    const float* lb = lam1 + (int64_t)b * NC * NVp + k0;
+    const int8_t* cls = cv.wcls + (int64_t)w * NVp + k0;
+    const float* vn = reinterpret_cast<const float*>(cv.wvn) + (int64_t)w * NVp + k0;
 #pragma unroll
-    for (int a = 0; a < DIM; ++a) {
-      const int q = fdiv_small_a(kk, inv_nv);
-      vel[e][a] = s_v[kk - q * nv];
-      kk = q;
+    for (int e = 0; e < 4; ++e) {
+      if (cls[e] != 0) continue;
+      ly[0][e] += r * (lb[e] + mu * vn[e]);
+      if (NC == 2) ly[NC - 1][e] += r * lb[NVp + e];
     }
   }
 }
 
-__device__ __forceinline__ void ld4f(const float* p, float v[4]) {
-  const float4 a = *reinterpret_cast<const float4*>(p);
-  v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-}
-__device__ __forceinline__ void st4f(float* p, const float v[4]) { *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]); }
-
-// lam_f~ at interior points from lam1, the wall terms and the relaxation VJP (FP32)
-template <int DIM>
-__global__ void __launch_bounds__(256) k_adj_relax_wp(CaseView cv, const float* FT, const double* amom, const float* lam1,
-                                                      const double* wmu, const int32_t* tslot, const int32_t* wall_of,
-                                                      float* LFT, double* dtheta) {
-  constexpr int NC = DIM == 2 ? 2 : 1;
+// lam_f~ at interior points from lam1, the wall terms and the relaxation VJP (FP32): one
+// warp per point, sums and outputs in packed FP32x2 pairs of velocities.  One dJ/dKn term
+// per CTA goes to the accumulator (one per point queued ten thousand additions to the same
+// address).  101^2 x 24^2: 62 us per launch, 74 with one velocity at a time; two chunks in
+// flight cost a CTA per SM (75 registers): 70 us.
+constexpr int ADJ_WARPS = 8;
+template <int DIM, bool ROW>
+__global__ void __launch_bounds__(32 * ADJ_WARPS) k_adj_relax_wp(CaseView cv, const float* FT, const double* amom,
+                                                                 const float* lam1, const double* wmu,
+                                                                 const int32_t* tslot, const int32_t* wall_of,
+                                                                 float* LFT, double* dtheta) {
+  constexpr int NC = DIM == 2 ? 2 : 1, NS = 4 + DIM;
   extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ double s_dk[ADJ_WARPS];
   const int W = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int cap = cv.cap, nv = cv.nv, NV = cv.NV, NVp = cv.NVp;
   float* s_v = reinterpret_cast<float*>(smem);
@@ -530,168 +556,169 @@ __global__ void __launch_bounds__(256) k_adj_relax_wp(CaseView cv, const float* 
   for (int q = threadIdx.x; q < nv; q += blockDim.x) s_v[q] = cv.vnodes_f[q];
   __syncthreads();
   const int t = blockIdx.x * W + warp;
-  if (t >= cv.n_int) return;
-  const int i = cv.int_idx[t];
-  const int m = cv.cnt[i];
-  // wall neighbours of i (usually none)
-  int nwb = 0;
-  for (int q0 = 0; q0 < m; q0 += 32) {
-    const int q = q0 + lane;
-    int b = -1, w = -1, sl = -1;
-    if (q < m) {
-      b = cv.col[(int64_t)i * cap + q];
-      w = wall_of[b];
-      sl = w >= 0 ? tslot[(int64_t)i * cap + q] : -1;
+  double dk = 0.0;
+  if (t < cv.n_int) {
+    const int i = cv.int_idx[t];
+    const int m = cv.cnt[i];
+    // wall neighbours of i (usually none)
+    int nwb = 0;
+    for (int q0 = 0; q0 < m; q0 += 32) {
+      const int q = q0 + lane;
+      int b = -1, w = -1, sl = -1;
+      if (q < m) {
+        b = cv.col[(int64_t)i * cap + q];
+        w = wall_of[b];
+        sl = w >= 0 ? tslot[(int64_t)i * cap + q] : -1;
+      }
+      const bool hit = w >= 0 && sl >= 0;
+      const unsigned bal = __ballot_sync(0xffffffffu, hit);
+      if (hit) {
+        const int pos = nwb + __popc(bal & ((1u << lane) - 1u));
+        s_wb[3 * pos] = b; s_wb[3 * pos + 1] = w; s_wb[3 * pos + 2] = sl;
+      }
+      nwb += __popc(bal);
     }
-    const bool hit = w >= 0 && sl >= 0;
-    const unsigned bal = __ballot_sync(0xffffffffu, hit);
-    if (hit) {
-      const int pos = nwb + __popc(bal & ((1u << lane) - 1u));
-      s_wb[3 * pos] = b; s_wb[3 * pos + 1] = w; s_wb[3 * pos + 2] = sl;
+    __syncwarp();
+    const double* mo = amom + (int64_t)i * MOM_STRIDE;
+    const float rho = (float)mo[0], T = (float)mo[4];
+    float U[DIM];
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) U[a] = (float)mo[1 + a];
+    const float wv = cv.wv_f;
+    const float R = rho / wv;
+    float tau = 0.0f, ca = 1.0f, cb = 0.0f, dadtau = 0.0f;
+    if (cv.tau_mode != 2) {
+      const float kn = cv.kn_f, dtf = cv.dt_f;
+      tau = cv.tau_mode == 1 ? 0.7978845608f * kn : 0.7978845608f * kn / (rho * sqrtf(T));
+      ca = tau / (tau + dtf);
+      cb = dtf / (tau + dtf);
+      dadtau = dtf / ((tau + dtf) * (tau + dtf));
     }
-    nwb += __popc(bal);
-  }
-  __syncwarp();
-  const double* mo = amom + (int64_t)i * MOM_STRIDE;
-  const float rho = (float)mo[0], T = (float)mo[4];
-  float U[DIM];
+    const float twopiT = 6.283185307f * T;
+    const float pref = DIM == 2 ? rho / twopiT : rho / (twopiT * sqrtf(twopiT));
+    const float nl2 = -0.5f / T;
+    const float inv_nv = 1.0f / (float)nv;
+    const int nchunk = NVp >> 2;
+    const int64_t rowlen = (int64_t)NC * NVp;
+    const float* l1 = lam1 + (int64_t)i * rowlen;
+    const float* ft = FT + (int64_t)i * rowlen;
+    float* lf = LFT + (int64_t)i * rowlen;
+    // sum lam_y f~, sum lm M (lm = lam_g + T lam_h), sum lm M |c|^2, sum lam_h M, sum lm M c
+    float2 cs[NS];
 #pragma unroll
-  for (int a = 0; a < DIM; ++a) U[a] = (float)mo[1 + a];
-  const float wv = cv.wv_f;
-  const float R = rho / wv;
-  float tau = 0.0f, ca = 1.0f, cb = 0.0f, dadtau = 0.0f;
-  if (cv.tau_mode != 2) {
-    const float kn = cv.kn_f, dtf = cv.dt_f;
-    tau = cv.tau_mode == 1 ? 0.7978845608f * kn : 0.7978845608f * kn / (rho * sqrtf(T));
-    ca = tau / (tau + dtf);
-    cb = dtf / (tau + dtf);
-    dadtau = dtf / ((tau + dtf) * (tau + dtf));
-  }
-  const float twopiT = 6.283185307f * T;
-  const float pref = DIM == 2 ? rho / twopiT : rho / (twopiT * sqrtf(twopiT));
-  const float nl2 = -0.5f / T;
-  const float inv_nv = 1.0f / (float)nv;
-  const int nchunk = NVp >> 2, nslice = (nchunk + 31) >> 5;
-  const int64_t rowlen = (int64_t)NC * NVp;
-  const float* l1 = lam1 + (int64_t)i * rowlen;
-  const float* ft = FT + (int64_t)i * rowlen;
-  float* lf = LFT + (int64_t)i * rowlen;
-  float cs[5 + DIM];
+    for (int q = 0; q < NS; ++q) cs[q] = f2(0.0f, 0.0f);
+    for (int chunk = lane; chunk < nchunk; chunk += 32) {
+      const int k0 = 4 * chunk;
+      float ly[NC][4], ftv[NC][4];
+      lam_y4<NC>(cv, l1, lam1, wmu, s_wb, nwb, k0, ly);
+      if (cv.tau_mode == 2) {
 #pragma unroll
-  for (int q = 0; q < 5 + DIM; ++q) cs[q] = 0.0f;
-  for (int sl = 0; sl < nslice; ++sl) {
-    const int chunk = sl * 32 + lane;
-    if (chunk >= nchunk) break;
-    const int k0 = 4 * chunk;
-    float vel[4][DIM];
-    bool kin[4];
-    chunk_vel_a<DIM>(k0, nv, NV, inv_nv, s_v, vel, kin);
-    float ly[NC][4], ftv[NC][4];
+        for (int c = 0; c < NC; ++c) st4(lf + (int64_t)c * NVp + k0, ly[c]);
+        continue;
+      }
 #pragma unroll
-    for (int c = 0; c < NC; ++c) { ld4f(l1 + (int64_t)c * NVp + k0, ly[c]); ld4f(ft + (int64_t)c * NVp + k0, ftv[c]); }
-    for (int q = 0; q < nwb; ++q) {
-      const int b = s_wb[3 * q], w = s_wb[3 * q + 1], slb = s_wb[3 * q + 2];
-      const float r = reinterpret_cast<const float*>(cv.recon)[(int64_t)b * cap + slb];
-      const float mu = (float)wmu[w];
-      const float* lb = lam1 + (int64_t)b * rowlen + k0;
-      const int8_t* cls = cv.wcls + (int64_t)w * NVp + k0;
-      const float* vn = reinterpret_cast<const float*>(cv.wvn) + (int64_t)w * NVp + k0;
+      for (int c = 0; c < NC; ++c) ld4(ft + (int64_t)c * NVp + k0, ftv[c]);
+      float vel[4][DIM];
+      bool kin[4];
+      chunk_velocities<DIM, 4, ROW>(k0, nv, NV, inv_nv, s_v, vel, kin);
+      if (!kin[3]) {
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        if (cls[e] != 0) continue;
-        ly[0][e] += r * (lb[e] + mu * vn[e]);
-        if (NC == 2) ly[NC - 1][e] += r * lb[NVp + e];
+        for (int e = 0; e < 4; ++e)
+#pragma unroll
+          for (int c = 0; c < NC; ++c) ly[c][e] = kin[e] ? ly[c][e] : 0.0f;
+      }
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        float2 cc[DIM], c2 = f2(0.0f, 0.0f);
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) {
+          cc[d] = __fadd2_rn(f2(vel[2 * q][d], vel[2 * q + 1][d]), f2(-U[d], -U[d]));
+          c2 = d == 0 ? __fmul2_rn(cc[d], cc[d]) : __ffma2_rn(cc[d], cc[d], c2);
+        }
+        const float2 M0 = f2(pref * __expf(nl2 * c2.x), pref * __expf(nl2 * c2.y));
+        const float2 g = f2(ly[0][2 * q], ly[0][2 * q + 1]);
+        cs[0] = __ffma2_rn(g, f2(ftv[0][2 * q], ftv[0][2 * q + 1]), cs[0]);
+        float2 lm = g;
+        if (NC == 2) {
+          const float2 h = f2(ly[NC - 1][2 * q], ly[NC - 1][2 * q + 1]);
+          cs[0] = __ffma2_rn(h, f2(ftv[NC - 1][2 * q], ftv[NC - 1][2 * q + 1]), cs[0]);
+          lm = __ffma2_rn(f2(T, T), h, lm);
+          cs[3] = __ffma2_rn(h, M0, cs[3]);
+        }
+        const float2 lmM = __fmul2_rn(lm, M0);
+        cs[1] = __fadd2_rn(cs[1], lmM);
+        cs[2] = __ffma2_rn(lmM, c2, cs[2]);
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) cs[4 + d] = __ffma2_rn(lmM, cc[d], cs[4 + d]);
       }
     }
-    if (cv.tau_mode == 2) {
+    if (cv.tau_mode != 2) {
+      float sum[NS];
 #pragma unroll
-      for (int c = 0; c < NC; ++c) st4f(lf + (int64_t)c * NVp + k0, ly[c]);
-      continue;
-    }
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      if (!kin[e]) continue;
-      float c2 = 0.0f;
-      float cc[DIM];
-#pragma unroll
-      for (int d = 0; d < DIM; ++d) { cc[d] = vel[e][d] - U[d]; c2 = fmaf(cc[d], cc[d], c2); }
-      const float M0 = pref * __expf(nl2 * c2);
-      cs[0] = fmaf(ly[0][e], ftv[0][e], cs[0]);
-      cs[1] = fmaf(ly[0][e], M0, cs[1]);
-      float lm = ly[0][e];
-      if (NC == 2) {
-        cs[0] = fmaf(ly[NC - 1][e], ftv[NC - 1][e], cs[0]);
-        cs[1] = fmaf(ly[NC - 1][e], T * M0, cs[1]);
-        lm = fmaf(T, ly[NC - 1][e], lm);
-        cs[4] = fmaf(ly[NC - 1][e], M0, cs[4]);
+      for (int q = 0; q < NS; ++q) sum[q] = warp_sum(cs[q].x + cs[q].y);
+      const float Dm = DIM == 2 ? 2.0f : 3.0f;
+      const float dLda = sum[0] - sum[1];
+      float g_rho = cb * sum[1] / rho;
+      float g_T = cb * (sum[2] / (2.0f * T * T) - Dm * sum[1] / (2.0f * T)) + cb * sum[3];
+      if (cv.tau_mode == 0) {
+        g_rho += dLda * dadtau * (-tau / rho);
+        g_T += dLda * dadtau * (-tau / (2.0f * T));
       }
-      const float lmM = lm * M0;
-      cs[2] += lmM;
-      cs[3] = fmaf(lmM, c2, cs[3]);
+      dk = (double)(dLda * dadtau * tau);
+      const float k0c = g_rho * wv - g_T * T / R, kc2 = g_T / (3.0f * R);
+      float gu[DIM];
 #pragma unroll
-      for (int d = 0; d < DIM; ++d) cs[5 + d] = fmaf(lmM, cc[d], cs[5 + d]);
+      for (int d = 0; d < DIM; ++d) gu[d] = cb * sum[4 + d] / T / R;
+      for (int chunk = lane; chunk < nchunk; chunk += 32) {
+        const int k0 = 4 * chunk;
+        float vel[4][DIM];
+        bool kin[4];
+        float ly[NC][4];
+        lam_y4<NC>(cv, l1, lam1, wmu, s_wb, nwb, k0, ly);  // again (cheaper than storing lam_y)
+        chunk_velocities<DIM, 4, ROW>(k0, nv, NV, inv_nv, s_v, vel, kin);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          float2 c2 = f2(0.0f, 0.0f), gs = f2(k0c, k0c);
+#pragma unroll
+          for (int d = 0; d < DIM; ++d) {
+            const float2 cc = __fadd2_rn(f2(vel[2 * q][d], vel[2 * q + 1][d]), f2(-U[d], -U[d]));
+            c2 = d == 0 ? __fmul2_rn(cc, cc) : __ffma2_rn(cc, cc, c2);
+            gs = __ffma2_rn(f2(gu[d], gu[d]), cc, gs);
+          }
+          const float2 o = __ffma2_rn(f2(ca, ca), f2(ly[0][2 * q], ly[0][2 * q + 1]), __ffma2_rn(f2(kc2, kc2), c2, gs));
+          ly[0][2 * q] = o.x; ly[0][2 * q + 1] = o.y;
+          if (NC == 2) {
+            const float2 oh = __ffma2_rn(f2(ca, ca), f2(ly[NC - 1][2 * q], ly[NC - 1][2 * q + 1]), f2(kc2, kc2));
+            ly[NC - 1][2 * q] = oh.x; ly[NC - 1][2 * q + 1] = oh.y;
+          }
+        }
+        if (!kin[3]) {
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+#pragma unroll
+            for (int c = 0; c < NC; ++c) ly[c][e] = kin[e] ? ly[c][e] : 0.0f;
+        }
+#pragma unroll
+        for (int c = 0; c < NC; ++c) st4(lf + (int64_t)c * NVp + k0, ly[c]);
+      }
     }
   }
   if (cv.tau_mode == 2) return;
-#pragma unroll
-  for (int q = 0; q < 5 + DIM; ++q) cs[q] = warp_sum(cs[q]);
-  const float Dm = DIM == 2 ? 2.0f : 3.0f;
-  const float dLda = cs[0] - cs[1];
-  float g_rho = cb * cs[2] / rho;
-  float g_T = cb * (cs[3] / (2.0f * T * T) - Dm * cs[2] / (2.0f * T)) + cb * cs[4];
-  if (cv.tau_mode == 0) {
-    g_rho += dLda * dadtau * (-tau / rho);
-    g_T += dLda * dadtau * (-tau / (2.0f * T));
-  }
-  if (lane == 0) atomicAdd(&dtheta[3], (double)(dLda * dadtau * tau) / cv.kn);
-  const float k0c = g_rho * wv - g_T * T / R, kc2 = g_T / (3.0f * R);
-  float gu[DIM];
-#pragma unroll
-  for (int d = 0; d < DIM; ++d) gu[d] = cb * cs[5 + d] / T / R;
-  for (int sl = 0; sl < nslice; ++sl) {
-    const int chunk = sl * 32 + lane;
-    if (chunk >= nchunk) break;
-    const int k0 = 4 * chunk;
-    float vel[4][DIM];
-    bool kin[4];
-    chunk_vel_a<DIM>(k0, nv, NV, inv_nv, s_v, vel, kin);
-    float ly[NC][4];
-#pragma unroll
-    for (int c = 0; c < NC; ++c) ld4f(l1 + (int64_t)c * NVp + k0, ly[c]);
-    for (int q = 0; q < nwb; ++q) {  // the wall terms of lam_y again (cheaper than storing lam_y)
-      const int b = s_wb[3 * q], w = s_wb[3 * q + 1], slb = s_wb[3 * q + 2];
-      const float r = reinterpret_cast<const float*>(cv.recon)[(int64_t)b * cap + slb];
-      const float mu = (float)wmu[w];
-      const float* lb = lam1 + (int64_t)b * rowlen + k0;
-      const int8_t* cls = cv.wcls + (int64_t)w * NVp + k0;
-      const float* vn = reinterpret_cast<const float*>(cv.wvn) + (int64_t)w * NVp + k0;
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        if (cls[e] != 0) continue;
-        ly[0][e] += r * (lb[e] + mu * vn[e]);
-        if (NC == 2) ly[NC - 1][e] += r * lb[NVp + e];
-      }
-    }
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      float c2 = 0.0f, gsum = k0c;
-#pragma unroll
-      for (int d = 0; d < DIM; ++d) {
-        const float cc = vel[e][d] - U[d];
-        c2 = fmaf(cc, cc, c2);
-        gsum = fmaf(gu[d], cc, gsum);
-      }
-      ly[0][e] = kin[e] ? fmaf(ca, ly[0][e], fmaf(kc2, c2, gsum)) : 0.0f;
-      if (NC == 2) ly[NC - 1][e] = kin[e] ? fmaf(ca, ly[NC - 1][e], kc2) : 0.0f;
-    }
-#pragma unroll
-    for (int c = 0; c < NC; ++c) st4f(lf + (int64_t)c * NVp + k0, ly[c]);
+  if (lane == 0) s_dk[warp] = dk;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double s = 0.0;
+    for (int w = 0; w < W; ++w) s += s_dk[w];
+    atomicAdd(&dtheta[3], s / cv.kn);
   }
 }
 
-// lam0 = L^T lam_f~ (FP32, warp per point, packed FP32x2 as in the forward transport)
-template <int DIM>
-__global__ void __launch_bounds__(256) k_adj_transport_wp(CaseView cv, const float* LFT, const float* SK, const int32_t* tslot, float* lam0) {
+// lam0 = L^T lam_f~ (FP32, one warp per point): with ROW (nv % 4 == 0) in the packed pairs
+// of the forward transport, four rows in flight, the 2D coefficients in one 16-byte load.
+// 101^2 x 24^2: 65 us per launch, 90 with one velocity at a time and 64-bit row indices.
+template <int DIM, bool ROW>
+__global__ void __launch_bounds__(128) k_adj_transport_wp(CaseView cv, const float* LFT, const float* SK,
+                                                          const int32_t* tslot, float* lam0) {
   constexpr int NC = DIM == 2 ? 2 : 1;
   constexpr int DD = DIM * DIM;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -728,51 +755,82 @@ __global__ void __launch_bounds__(256) k_adj_transport_wp(CaseView cv, const flo
   }
   __syncwarp();
   const float inv_nv = 1.0f / (float)nv;
-  const int nchunk = NVp >> 2, nslice = (nchunk + 31) >> 5;
+  const int nchunk = NVp >> 2;
   const int64_t rowlen = (int64_t)NC * NVp;
+  const uint32_t rb = (uint32_t)(NC * NVp * 4);  // bytes of a row
   const float two_dt = cv.two_dt_f;
-  for (int sl = 0; sl < nslice; ++sl) {
-    const int chunk = sl * 32 + lane;
-    if (chunk >= nchunk) break;
+  for (int chunk = lane; chunk < nchunk; chunk += 32) {
     const int k0 = 4 * chunk;
     float vel[4][DIM];
     bool kin[4];
-    chunk_vel_a<DIM>(k0, nv, NV, inv_nv, s_v, vel, kin);
+    chunk_velocities<DIM, 4, ROW>(k0, nv, NV, inv_nv, s_v, vel, kin);
     float diag[4] = {0.0f, 0.0f, 0.0f, 0.0f}, acc[NC][4];
-    if (interior) ld4f(SK + (int64_t)p * NVp + k0, diag);
+    if (interior) ld4(SK + (int64_t)p * NVp + k0, diag);
+    const float* l0 = LFT + k0;
+    const float* l1 = l0 + NVp;
+    if constexpr (ROW) {
+      const float2 cx[2] = {f2(vel[0][0], vel[1][0]), f2(vel[2][0], vel[3][0])};
+      float crest[DIM - 1];
 #pragma unroll
-    for (int c = 0; c < NC; ++c)
+      for (int a = 1; a < DIM; ++a) crest[a - 1] = vel[0][a];
+      float2 skp[2] = {f2(0.0f, 0.0f), f2(0.0f, 0.0f)}, ap[NC][2];  // (skp: not used)
 #pragma unroll
-      for (int e = 0; e < 4; ++e) acc[c][e] = 0.0f;
-    for (int t = 0; t < mt; ++t) {
-      const int i = s_i[t];
-      float li[NC][4];
+      for (int c = 0; c < NC; ++c) { ap[c][0] = f2(0.0f, 0.0f); ap[c][1] = f2(0.0f, 0.0f); }
+#pragma unroll 4
+      for (int t = 0; t < mt; ++t) {
+        const int i = s_i[t];
+        float li[NC][4], P[DD];
 #pragma unroll
-      for (int c = 0; c < NC; ++c) ld4f(LFT + (int64_t)i * rowlen + (int64_t)c * NVp + k0, li[c]);
+        for (int c = 0; c < NC; ++c) ld4_ro(row_at(c ? l1 : l0, i, rb), li[c]);
+        if constexpr (DIM == 2) {
+          const float4 a = reinterpret_cast<const float4*>(s_P)[t];
+          P[0] = a.x; P[1] = a.y; P[2] = a.z; P[3] = a.w;
+        } else {
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        float mk = 0.0f;
-#pragma unroll
-        for (int d = 0; d < DIM; ++d) {
-          float pd = vel[e][0] * s_P[t * DD + d * DIM];
-#pragma unroll
-          for (int a = 1; a < DIM; ++a) pd = fmaf(vel[e][a], s_P[t * DD + d * DIM + a], pd);
-          mk += fminf(pd, 0.0f);
+          for (int q = 0; q < DD; ++q) P[q] = s_P[t * DD + q];
         }
+        row_upwind<DIM, NC, 2>(cx, crest, P, li, skp, ap);
+      }
 #pragma unroll
-        for (int c = 0; c < NC; ++c) acc[c][e] = fmaf(mk, li[c][e], acc[c][e]);
+      for (int c = 0; c < NC; ++c) {
+        acc[c][0] = ap[c][0].x; acc[c][1] = ap[c][0].y; acc[c][2] = ap[c][1].x; acc[c][3] = ap[c][1].y;
+      }
+    } else {
+#pragma unroll
+      for (int c = 0; c < NC; ++c)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[c][e] = 0.0f;
+#pragma unroll 2
+      for (int t = 0; t < mt; ++t) {
+        const int i = s_i[t];
+        float li[NC][4];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) ld4_ro(row_at(c ? l1 : l0, i, rb), li[c]);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          float mk = 0.0f;
+#pragma unroll
+          for (int d = 0; d < DIM; ++d) {
+            float pd = vel[e][0] * s_P[t * DD + d * DIM];
+#pragma unroll
+            for (int a = 1; a < DIM; ++a) pd = fmaf(vel[e][a], s_P[t * DD + d * DIM + a], pd);
+            mk += fminf(pd, 0.0f);
+          }
+#pragma unroll
+          for (int c = 0; c < NC; ++c) acc[c][e] = fmaf(mk, li[c][e], acc[c][e]);
+        }
       }
     }
     float own[NC][4], out[NC][4];
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-      if (interior) ld4f(LFT + (int64_t)p * rowlen + (int64_t)c * NVp + k0, own[c]);
+      if (interior) ld4(LFT + (int64_t)p * rowlen + (int64_t)c * NVp + k0, own[c]);
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         const float l = interior ? own[c][e] : 0.0f;
         out[c][e] = kin[e] ? l + two_dt * (diag[e] * l - acc[c][e]) : 0.0f;
       }
-      st4f(lam0 + (int64_t)p * rowlen + (int64_t)c * NVp + k0, out[c]);
+      st4(lam0 + (int64_t)p * rowlen + (int64_t)c * NVp + k0, out[c]);
     }
   }
 }
@@ -787,30 +845,32 @@ int launch_adjoint_fp32(const CaseView& cv0, const void* lam1, void* lam0, doubl
   cv.sk_out = SK;
   cv.mom = amom;
   int n = launch_transport_fp32(cv, s);
-  const int W = 8;
   if (cv.n_wall > 0) {
     if (cv.dim == 2) k_adj_walls<float, 2><<<cv.n_wall, 256, 0, s>>>(cv, (const float*)Y, (const float*)lam1, wmu, dtheta);
     else k_adj_walls<float, 3><<<cv.n_wall, 256, 0, s>>>(cv, (const float*)Y, (const float*)lam1, wmu, dtheta);
     ++n;
   }
+  const bool row = cv.nv % 4 == 0;
   if (cv.n_int > 0) {
+    const int W = ADJ_WARPS, grid = (cv.n_int + W - 1) / W;
     const size_t smem = 256 + sizeof(int32_t) * (size_t)cv.cap * 3 * W;
-    const int grid = (cv.n_int + W - 1) / W;
-    if (cv.dim == 2) k_adj_relax_wp<2><<<grid, 32 * W, smem, s>>>(cv, (const float*)FT, amom, (const float*)lam1, wmu, tslot, wall_of, (float*)LFT, dtheta);
-    else k_adj_relax_wp<3><<<grid, 32 * W, smem, s>>>(cv, (const float*)FT, amom, (const float*)lam1, wmu, tslot, wall_of, (float*)LFT, dtheta);
+    auto go = [&](auto k) {
+      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      k<<<grid, 32 * W, smem, s>>>(cv, (const float*)FT, amom, (const float*)lam1, wmu, tslot, wall_of, (float*)LFT, dtheta);
+    };
+    if (cv.dim == 2) row ? go(k_adj_relax_wp<2, true>) : go(k_adj_relax_wp<2, false>);
+    else row ? go(k_adj_relax_wp<3, true>) : go(k_adj_relax_wp<3, false>);
     ++n;
   }
   {
-    const int DD = cv.dim * cv.dim;
+    const int W = 4, DD = cv.dim * cv.dim, grid = (cv.n + W - 1) / W;
     const size_t smem = 256 + sizeof(float) * (size_t)W * cv.cap * DD + sizeof(int32_t) * (size_t)W * cv.cap;
-    const int grid = (cv.n + W - 1) / W;
-    if (cv.dim == 2) {
-      cudaFuncSetAttribute(k_adj_transport_wp<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      k_adj_transport_wp<2><<<grid, 32 * W, smem, s>>>(cv, (const float*)LFT, SK, tslot, (float*)lam0);
-    } else {
-      cudaFuncSetAttribute(k_adj_transport_wp<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      k_adj_transport_wp<3><<<grid, 32 * W, smem, s>>>(cv, (const float*)LFT, SK, tslot, (float*)lam0);
-    }
+    auto go = [&](auto k) {
+      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      k<<<grid, 32 * W, smem, s>>>(cv, (const float*)LFT, SK, tslot, (float*)lam0);
+    };
+    if (cv.dim == 2) row ? go(k_adj_transport_wp<2, true>) : go(k_adj_transport_wp<2, false>);
+    else row ? go(k_adj_transport_wp<3, true>) : go(k_adj_transport_wp<3, false>);
     ++n;
   }
   return n;
