@@ -17,8 +17,13 @@ namespace bgk {
 //   3D: 2 (27^3 x 12^3 ALE: 1 / 2 / 3 / 4 rows 944 / 834 / 847 / 834 us);
 //   mirror pairs (two rows per neighbour): 5 at 16 warps per SM (41^3 x 16^3: 2 / 4 / 5 / 6
 //   / 8 neighbours 5.76 / 5.07 / 4.96 / 5.00 / 4.98 ms; 5.33 ms at best with 24 warps).
-template <int DIM, bool ROW>
-__host__ __device__ constexpr int nbr_unroll() { return DIM == 2 && ROW ? 4 : 2; }
+//   2D, shared grid row, a slab of the velocity grid in FP32: 2 (step of the 201^2 x 32^2
+//   ALE case in 1 slab: 1 / 2 / 3 / 4 rows 0.620 / 0.543 / 0.566 / 0.556 ms; in 4 slabs
+//   0.954 / 0.885 / 0.909 / 0.901); BF16 keeps 4 (2 slabs: 0.688 / 0.648 / 0.652 / 0.639).
+template <typename S, int DIM, bool ROW, bool SH>
+__host__ __device__ constexpr int nbr_unroll() {
+  return DIM == 2 && ROW && !(SH && sizeof(S) == 4) ? 4 : 2;
+}
 constexpr int kMirrorUnroll = 5;
 
 // ---------------------------------------------------------------------------
@@ -616,7 +621,7 @@ __device__ __forceinline__ void transport_point_wp(const CaseView& cv, const int
         for (int c = 0; c < NC; ++c) ldv_ro<S, VPL>(row_at(c ? fj1 : fj0, j, rb), fv[c]);
         row_upwind<DIM, NC, NP>(cx, crest, P, fv, skp, ap);
       };
-#pragma unroll (nbr_unroll<DIM, true>())
+#pragma unroll (nbr_unroll<S, DIM, true, SH>())
       for (int s = 0; s < ms; ++s) {
         float P[DD];
         const int j = staged_nbr<DIM>(s_P, s_col, s, P);
@@ -681,7 +686,7 @@ __device__ __forceinline__ void transport_point_wp(const CaseView& cv, const int
           for (int c = 0; c < NC; ++c) ap[c][q] = __ffma2_rn(mk[q], f2(fv[c][2 * q], fv[c][2 * q + 1]), ap[c][q]);
         }
       };
-#pragma unroll (nbr_unroll<DIM, false>())
+#pragma unroll (nbr_unroll<S, DIM, false, SH>())
       for (int s = 0; s < ms; ++s) {
         float P[DD];
         const int j = staged_nbr<DIM>(s_P, s_col, s, P);
