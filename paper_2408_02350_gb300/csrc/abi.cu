@@ -3,8 +3,8 @@
 // One time step of a case (Sec. 3.2, read in the order neighbours/stencils ->
 // transport -> moments -> relaxation -> walls -> motion):
 //   [ale or first step] cell lists, neighbour lists, WLS stencils
-//   k_transport   f[cur] -> f[1-cur] at interior points (transport, moments, relaxation)
-//   k_walls       f[1-cur] at wall points (reconstruction + diffuse reflection)
+//   transport     f[cur] -> f[1-cur] at interior points (transport, moments, relaxation)
+//   walls         f[1-cur] at wall points (reconstruction + diffuse reflection)
 //   [ale]         k_move: x += dt U^{n+1}
 // All launches go to the caller's stream; nothing synchronises inside bgk_step.
 #include <cuda_runtime.h>
