@@ -723,7 +723,7 @@ int bgk_init(const bgk_params* p, int32_t n_cases, const int64_t* n_points, cons
     if (q.skin > 0) {
       // candidate capacity: max_nbrs scaled by the volume ratio of the two radii, plus 10 %
       const double r = std::pow(1.0 + q.skin, dim) * 1.1;
-      v.ccap = (int32_t)std::min<double>(std::ceil(v.cap * r), 4096.0);
+      v.ccap = (int32_t)std::min<double>(std::ceil(v.cap * r), MAX_CANDIDATES);
       if ((st = dalloc(ctx, &v.xb, ncap * dim))) return bail(st);
       if ((st = dalloc(ctx, &v.ccnt, ncap))) return bail(st);
       if ((st = dalloc(ctx, &v.ccol, (size_t)ncap * v.ccap))) return bail(st);

@@ -43,6 +43,9 @@ struct DevStatus {
 // Moments are stored per point as MOM_STRIDE doubles: rho, U[3], T.
 constexpr int MOM_STRIDE = 5;
 
+// Largest candidate-list capacity of a case with skin lists.
+constexpr int MAX_CANDIDATES = 4096;
+
 // Everything a kernel needs about one case, passed by value.  All pointers are
 // device pointers owned by the context.
 struct CaseView {

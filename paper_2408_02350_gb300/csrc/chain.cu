@@ -159,9 +159,10 @@ int launch_chain(const CaseView& cv, int* grid_cache, long long max_spins, cudaS
   const size_t smem = sizeof(int32_t) * (size_t)cv.ccap * CHAIN_WARPS;
   const void* fn = cv.dim == 2 ? (const void*)k_chain<2> : (const void*)k_chain<3>;
   if (*grid_cache <= 0) {
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-      return -1;
+    // the same limit for every case (128 KB): the attribute belongs to the kernel, so a
+    // case that set its own size would take it from the larger cases of the process
+    constexpr int limit = sizeof(int32_t) * MAX_CANDIDATES * CHAIN_WARPS;
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, limit) != cudaSuccess) return -1;
     int dev = 0, nsm = 0, coop = 0, per_sm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
