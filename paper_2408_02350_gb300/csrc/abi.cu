@@ -103,6 +103,7 @@ struct CaseHost {
   cudaEvent_t ev_recon[2] = {nullptr, nullptr};
   int64_t chain = 0;
   int chain_grid = 0;  // CTAs of the cooperative side-chain kernel (0: not yet sized)
+  bool chain_refused = false;  // its launch was refused: the separate kernels from then on
   int64_t cap_n = 0;  // capacity of the per-point arrays (initial points + spare_points)
   // point management scratch (allocated on first use, cap_n entries)
   int32_t *pm_nn = nullptr, *pm_role = nullptr, *pm_newidx = nullptr, *pm_addidx = nullptr, *pm_totals = nullptr;
@@ -387,26 +388,28 @@ int move_and_prebuild(bgk_ctx* ctx, CaseHost& c, cudaStream_t s) {
   nx.col = c.nx_col;
   nx.P = c.nx_P;
   nx.recon = c.nx_recon;
-  if (chain_eligible(nx)) {
+  bool chained = false;
+  if (chain_eligible(nx) && !c.chain_refused) {
     // motion, lists and interior stencils in one cooperative launch (timed as lists)
     if ((st = timed_begin(ctx, K_NBR, q, &e))) return st;
     const int k = launch_chain(nx, &c.chain_grid, ctx->watchdog, q);
-    if (k < 0) return fail(ctx, BGK_E_CUDA, "cooperative launch of the side chain failed");
-    ctx->launches += k;
+    chained = k > 0;
+    c.chain_refused = !chained;
+    if (chained) ctx->launches += k;
     CKL(ctx);
     if ((st = timed_end(ctx, e, q))) return st;
-    if (nx.wls_order == 2) {
-      if ((st = timed_begin(ctx, K_STENCIL, q, &e))) return st;
-      ctx->launches += launch_stencils(nx, q, 1);
-      CKL(ctx);
-      if ((st = timed_end(ctx, e, q))) return st;
-    }
-  } else {
+  }
+  if (!chained) {
     if ((st = timed_begin(ctx, K_MOVE, q, &e))) return st;
     ctx->launches += launch_move(c.cv, q);
     CKL(ctx);
     if ((st = timed_end(ctx, e, q))) return st;
     if ((st = build_lists_into(ctx, nx, q, 1))) return st;
+  } else if (nx.wls_order == 2) {
+    if ((st = timed_begin(ctx, K_STENCIL, q, &e))) return st;
+    ctx->launches += launch_stencils(nx, q, 1);
+    CKL(ctx);
+    if ((st = timed_end(ctx, e, q))) return st;
   }
   CK(ctx, cudaEventRecord(c.ev_join, q));
   if ((st = timed_begin(ctx, K_STENCIL, q, &e))) return st;

@@ -152,9 +152,10 @@ int launch_manage_apply(const CaseView& cv, int64_t cap_n, const int32_t* nn, co
 int launch_neighbours_skin(const CaseView& cv, cudaStream_t s);
 // ALE with a skin, FP32/BF16 storage: motion, candidate rebuild when due, filter and
 // interior stencils (the linear fit; the second-order fit is launched after it) of the
-// list set in cv as one cooperative launch (grid size cached in *grid_cache); returns 1, or -1 when the cooperative launch is unavailable.  A grid
-// barrier waits at most max_spins polls (0: about a second), then the kernel records
-// ST_TIMEOUT and its CTAs return.
+// list set in cv as one cooperative launch (grid size cached in *grid_cache); returns 1,
+// or -1 when the cooperative launch is refused (nothing has run: the separate kernels give
+// the same lists).  A grid barrier waits at most max_spins polls (0: about a second), then
+// the kernel records ST_TIMEOUT and its CTAs return.
 bool chain_eligible(const CaseView& cv);
 int launch_chain(const CaseView& cv, int* grid_cache, long long max_spins, cudaStream_t s);
 // Velocity-sharded step (slabs of the velocity grid, coupled only through velocity sums;

@@ -154,8 +154,13 @@ bool chain_eligible(const CaseView& cv) { return cv.ale && cv.sk && cv.storage !
 #ifndef BGK_CHAIN_PER_SM
 #define BGK_CHAIN_PER_SM 2
 #endif
+// Times the co-resident grid (1; a larger one is refused by the runtime, for the test of
+// the separate kernels that then run).
+#ifndef BGK_CHAIN_GRID_SCALE
+#define BGK_CHAIN_GRID_SCALE 1
+#endif
 
-int launch_chain(const CaseView& cv, int* grid_cache, long long max_spins, cudaStream_t s) {
+static int try_chain(const CaseView& cv, int* grid_cache, long long max_spins, cudaStream_t s) {
   const size_t smem = sizeof(int32_t) * (size_t)cv.ccap * CHAIN_WARPS;
   const void* fn = cv.dim == 2 ? (const void*)k_chain<2> : (const void*)k_chain<3>;
   if (*grid_cache <= 0) {
@@ -170,7 +175,7 @@ int launch_chain(const CaseView& cv, int* grid_cache, long long max_spins, cudaS
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, CHAIN_THREADS, smem) != cudaSuccess || per_sm < 1)
       return -1;
     if (BGK_CHAIN_PER_SM > 0 && per_sm > BGK_CHAIN_PER_SM) per_sm = BGK_CHAIN_PER_SM;
-    *grid_cache = nsm * per_sm;
+    *grid_cache = nsm * per_sm * BGK_CHAIN_GRID_SCALE;
   }
   const double half = 0.5 * cv.h * cv.skin;
   double thr2 = half * half * (1.0 - 1e-6);
@@ -183,6 +188,12 @@ int launch_chain(const CaseView& cv, int* grid_cache, long long max_spins, cudaS
   if (cudaLaunchCooperativeKernel(fn, dim3(*grid_cache), dim3(CHAIN_THREADS), args, smem, s) != cudaSuccess)
     return -1;
   return 1;
+}
+
+int launch_chain(const CaseView& cv, int* grid_cache, long long max_spins, cudaStream_t s) {
+  const int k = try_chain(cv, grid_cache, max_spins, s);
+  if (k < 0) cudaGetLastError();  // a refusal is not the error of the launch that follows
+  return k;
 }
 
 }  // namespace bgk

@@ -1,11 +1,17 @@
 """The side chain of moving-point steps (motion, lists and stencils of the next step as one
-cooperative launch): contexts of different sizes side by side."""
+cooperative launch): contexts of different sizes side by side, and a launch that the runtime
+refuses."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
 import bgk_inputs as bi
 
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 @pytest.fixture(scope="module")
@@ -46,3 +52,42 @@ def test_contexts_with_different_candidate_capacities_step_in_turn(g, wls):
         s.sync()
         assert np.array_equal(s.get_f(0, np.float32), f) and np.array_equal(s.positions(), x)
         s.close()
+
+
+# The cases below step in a process of their own (argv: library, output folder).
+_REFUSED = [{"wls_order": 1}, {"wls_order": 2}, {"wls_order": 2, "storage": "bf16"}, {"body": True, "n": 41}]
+_STEP = r"""
+import sys
+import numpy as np
+sys.path.insert(0, %(root)r)
+import bgk_inputs as bi
+import paper_2408_02350_gb300 as g
+g.LIB_PATH = sys.argv[1]
+for k, over in enumerate(%(cases)r):
+    over = dict(over)
+    name = "body2d_ale_n201_v32_f32" if over.pop("body", False) else "cavity2d_ale_n201_v32_f32"
+    p = bi.config(name, **dict(dict(n=21, nv=8, vmax=4.0), **over))
+    s = g.Solver([p], [bi.cloud_for(p)])
+    s.set_maxwellian()
+    s.step(5)
+    s.sync()
+    np.savez(sys.argv[2] + "/%%d.npz" %% k, f=s.get_f(), x=s.positions(), n=s.stats()["launches"])
+    s.close()
+"""
+
+
+def test_a_refused_cooperative_launch_falls_back_to_the_separate_kernels(g, tmp_path):
+    # a build whose cooperative grid is 64 times what fits: the runtime refuses the launch
+    # (an error code, nothing runs); the separate kernels then give the same bits
+    from paper_2408_02350_gb300 import _build
+    big = _build._build_into(str(tmp_path / "build"), str(tmp_path / "libbgk_big.so"), False, False,
+                             ["-DBGK_CHAIN_GRID_SCALE=64"])
+    for tag, lib in (("a", _build.lib_path()), ("b", big)):
+        os.makedirs(str(tmp_path / tag))
+        r = subprocess.run([sys.executable, "-c", _STEP % {"root": ROOT, "cases": _REFUSED}, lib, str(tmp_path / tag)],
+                           capture_output=True, text=True, timeout=600)
+        assert r.returncode == 0, r.stderr[-2000:]
+    for k in range(len(_REFUSED)):
+        a, b = np.load(str(tmp_path / ("a/%d.npz" % k))), np.load(str(tmp_path / ("b/%d.npz" % k)))
+        assert np.array_equal(a["f"], b["f"]) and np.array_equal(a["x"], b["x"]), k
+        assert b["n"] > a["n"], k
