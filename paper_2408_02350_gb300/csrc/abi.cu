@@ -1283,8 +1283,9 @@ int bgk_sync(bgk_ctx* ctx, void* stream) {
         c.next_ready = false;
       }
     }
-    // the first condition in this order (bounds, overflow, singular, non-finite, timeout)
-    // is the return code; the text names every one
+    // the first condition in this order (bounds, overflow, timeout, singular, non-finite)
+    // is the return code; the text names every one.  Lists that a timeout cut short may
+    // leave rows empty, whose stencils are then singular: the timeout is the cause.
     char all[96];
     snprintf(all, sizeof(all), " (device flags:%s%s%s%s%s)", hs.flags & ST_BOUNDS ? " bounds" : "",
              hs.flags & ST_OVERFLOW ? " overflow" : "", hs.flags & ST_SINGULAR ? " singular" : "",
@@ -1292,11 +1293,11 @@ int bgk_sync(bgk_ctx* ctx, void* stream) {
     if (hs.flags & ST_BOUNDS)
       return fail(ctx, BGK_E_BOUNDS, "an index outside the point range was found and skipped%s", all);
     if (hs.flags & ST_OVERFLOW) return fail(ctx, BGK_E_NBR_OVERFLOW, "a point has more than max_nbrs neighbours%s", all);
+    if (hs.flags & ST_TIMEOUT) return fail(ctx, BGK_E_TIMEOUT, "a bounded device wait gave up%s", all);
     if (hs.flags & ST_SINGULAR)
       return fail(ctx, BGK_E_SINGULAR, "singular WLS system (too few or degenerate neighbours)%s", all);
     if (hs.flags & ST_NONFINITE)
       return fail(ctx, BGK_E_NONFINITE, "non-finite or non-positive density or temperature%s", all);
-    if (hs.flags & ST_TIMEOUT) return fail(ctx, BGK_E_TIMEOUT, "a bounded device wait gave up%s", all);
   }
   return BGK_OK;
 }

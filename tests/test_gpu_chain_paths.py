@@ -1,6 +1,6 @@
 """The side chain of moving-point steps (motion, lists and stencils of the next step as one
-cooperative launch): contexts of different sizes side by side, and a launch that the runtime
-refuses."""
+cooperative launch): contexts of different sizes side by side, a launch that the runtime
+refuses, and a wait that gives up before any list is there."""
 import os
 import subprocess
 import sys
@@ -91,3 +91,28 @@ def test_a_refused_cooperative_launch_falls_back_to_the_separate_kernels(g, tmp_
         a, b = np.load(str(tmp_path / ("a/%d.npz" % k))), np.load(str(tmp_path / ("b/%d.npz" % k)))
         assert np.array_equal(a["f"], b["f"]) and np.array_equal(a["x"], b["x"]), k
         assert b["n"] > a["n"], k
+
+
+@pytest.mark.parametrize("wls,storage", [(1, "f32"), (2, "f32"), (2, "bf16")])
+def test_timeout_on_the_first_step_is_reported_as_such(g, wls, storage):
+    # one poll per wait: the rows of the next step's lists that no CTA reached are empty,
+    # and their stencils and wall weights singular in consequence; the run then continues
+    # as one without a timeout
+    p = _ale(wls_order=wls, storage=storage, n=41)
+    ref = g.Solver([p], [bi.cloud_for(p)])
+    ref.set_maxwellian()
+    ref.step(6)
+    ref.sync()
+    s = g.Solver([p], [bi.cloud_for(p)])
+    s.set_maxwellian()
+    g.bgk_set_watchdog(s.ctx, 1)
+    s.step(1)
+    with pytest.raises(g.BGKError) as e:
+        s.sync()
+    assert e.value.code == g.BGK_E_TIMEOUT
+    g.bgk_set_watchdog(s.ctx, 0)
+    s.step(5)
+    s.sync()
+    assert np.array_equal(s.get_f(), ref.get_f()) and np.array_equal(s.positions(), ref.positions())
+    s.close()
+    ref.close()
