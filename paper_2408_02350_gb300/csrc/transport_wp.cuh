@@ -87,10 +87,13 @@ __device__ __forceinline__ void chunk_velocities(int k0, int nv, int NV, float i
 }
 
 __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
-// 2^x by the hardware's approximate base-2 exponential (relative error about 2^-22).
+// 2^x by the hardware's approximate base-2 exponential (relative error about 2^-22).  FTZ:
+// results below 2^-126 are zero; without it they come as subnormal numbers.
+template <bool FTZ>
 __device__ __forceinline__ float exp2_approx(float x) {
   float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  if (FTZ) asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  else asm("ex2.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
 __device__ __forceinline__ float2 min0(float2 p) { return make_float2(fminf(p.x, 0.0f), fminf(p.y, 0.0f)); }
@@ -376,7 +379,8 @@ __device__ __forceinline__ void relax_point(const CaseView& cv, const int i, con
     for (int c = 0; c < NC; ++c) ldv<S, VPL>(fo + (int64_t)c * NVp + k0, ft[c]);
     if constexpr (ROW || packed_ragged<S>()) {
       // in packed pairs: |v - U|^2 (ROW: (v_x - U_x)^2 + r2, r2 shared by the lane's
-      // velocities); M from 2^(l2 |v - U|^2), l2 = -log2(e) / (2 T)
+      // velocities); M from 2^(l2 |v - U|^2), l2 = -log2(e) / (2 T), its tails below 2^-126
+      // kept on ragged grids
       float r2 = 0.0f;
       if (ROW) {
 #pragma unroll
@@ -397,7 +401,7 @@ __device__ __forceinline__ void relax_point(const CaseView& cv, const int i, con
         }
         const float2 dx = __fadd2_rn(f2(vel[2 * q][0], vel[2 * q + 1][0]), f2(-Un[0], -Un[0]));
         const float2 ea = __fmul2_rn(__ffma2_rn(dx, dx, c2), f2(l2, l2));
-        const float2 bM = __fmul2_rn(f2(pref, pref), f2(exp2_approx(ea.x), exp2_approx(ea.y)));
+        const float2 bM = __fmul2_rn(f2(pref, pref), f2(exp2_approx<ROW>(ea.x), exp2_approx<ROW>(ea.y)));
         const float2 o0 = __ffma2_rn(f2(ca, ca), f2(ft[0][2 * q], ft[0][2 * q + 1]), bM);
         out[0][2 * q] = o0.x; out[0][2 * q + 1] = o0.y;
         if (NC == 2) {
