@@ -40,6 +40,9 @@ struct DevStatus {
 
 };
 
+// SMs of the GB300: sizes grids and groups of points only (speed, not results).
+constexpr int TARGET_SMS = 152;
+
 // Moments are stored per point as MOM_STRIDE doubles: rho, U[3], T.
 constexpr int MOM_STRIDE = 5;
 

@@ -1110,29 +1110,35 @@ __global__ void k_moments(CaseView cv, const S* f) {
   }
 }
 
-// FP32/BF16 storage: each warp streams MOM_GP consecutive points in turn, each lane 4
+// FP32/BF16 storage: each warp streams gp consecutive points in turn, each lane 4
 // consecutive velocities per chunk (16-byte loads, eight chunks in flight, velocity nodes
 // staged in shared memory as FP32) into Kahan-compensated FP32 sums.  A point's lane sums
 // are reduced across the warp as FP32 pairs with exact high-part additions (no FP64 on
-// the 32-lane path); once the warp has all its points, lane g converts point g's pair
-// totals to FP64 and forms rho, U, T in FP64, so each FP64 instruction serves MOM_GP
-// points (FP64 runs at a small fraction of the FP32 rate).  SH: the raw sums of the
-// velocity slab (in FP64) to the exchange buffer instead.
-constexpr int MOM_GP = 8, MOM_WARPS = 4;  // points per warp (at most), warps per CTA
+// the 32-lane path); once the CTA has all its points, thread t converts point t's pair
+// totals to FP64 and forms rho, U, T in FP64, so each FP64 instruction serves up to 32
+// points (FP64 runs at a small fraction of the FP32 rate, whatever the lanes in use).  SH:
+// the raw sums of the velocity slab (in FP64) to the exchange buffer instead.  48 registers
+// (5 CTAs per SM), chosen so that the loads of a chunk stay in flight (left to the compiler,
+// 40 for BF16: 35 against 29 us, 41^2 x 63^2).
+constexpr int MOM_GP = 8, MOM_WARPS = 8;  // points per warp, warps per CTA (at most)
 // Points per warp: MOM_GP where that still gives every SM 32 warps, fewer for smaller
 // clouds (8 points per warp left 8 warps per SM on 101^2 points: 32 us for 47 MB).
-static int moments_gp(int n) { return std::max(1, std::min(MOM_GP, n / (152 * 32))); }
+static int moments_gp(int n) { return std::max(1, std::min(MOM_GP, n / (TARGET_SMS * 32))); }
+// Warps per CTA: 8, so that the FP64 part serves 8 points or more at once (21^3 points x 3^3
+// velocities, upload and moments: 17 us; 39 us with a warp for each point's FP64 part, 19 us
+// with 8 points per warp); 4 where the warps do not fill the SMs and 8 would spread them
+// unevenly.
+static int moments_warps(int n) { return n < TARGET_SMS * 32 ? MOM_WARPS / 2 : MOM_WARPS; }
 template <typename S, int DIM, bool ROW, bool SH = false>
-__global__ void __launch_bounds__(32 * MOM_WARPS) k_moments_wp(CaseView cv, const S* f, const int gp) {
+__global__ void __launch_bounds__(32 * MOM_WARPS, 5) k_moments_wp(CaseView cv, const S* f, const int gp) {
   constexpr int NC = DIM == 2 ? 2 : 1, VPL = 4, NQ = DIM + 2;
   __shared__ __align__(16) float s_v[64];  // chunk_velocities reads groups of 4
-  __shared__ float2 s_tot[MOM_WARPS][MOM_GP][NQ];
+  __shared__ float2 s_tot[MOM_WARPS * MOM_GP][NQ];
   for (int t = threadIdx.x; t < cv.nv; t += blockDim.x) s_v[t] = cv.vnodes_f[t];
   __syncthreads();
   const int W = blockDim.x >> 5, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int i0 = (blockIdx.x * W + warp) * gp;
-  if (i0 >= cv.n) return;
-  const int np = min(gp, cv.n - i0);
+  const int b0 = blockIdx.x * W * gp, i0 = b0 + warp * gp;
+  const int np = min(gp, cv.n - i0);  // (none or negative in the last CTA's idle warps)
   const int nv = cv.nv, NV = cv.NV, NVp = cv.NVp;
   const int vk0 = SH ? cv.vk0 : 0;
   const float inv_nv = 1.0f / (float)nv;
@@ -1178,15 +1184,15 @@ __global__ void __launch_bounds__(32 * MOM_WARPS) k_moments_wp(CaseView cv, cons
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1)
         pair_add(hi, lo, __shfl_xor_sync(0xffffffffu, hi, o), __shfl_xor_sync(0xffffffffu, lo, o));
-      if (lane == 0) s_tot[warp][g][q] = make_float2(hi, lo);
+      if (lane == 0) s_tot[warp * gp + g][q] = make_float2(hi, lo);
     }
   }
-  __syncwarp();
-  if (lane >= np) return;
-  const int i = i0 + lane;
+  __syncthreads();
+  const int i = b0 + threadIdx.x;
+  if (threadIdx.x >= W * gp || i >= cv.n) return;
   double tot[NQ];
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) tot[q] = (double)s_tot[warp][lane][q].x + (double)s_tot[warp][lane][q].y;
+  for (int q = 0; q < NQ; ++q) tot[q] = (double)s_tot[threadIdx.x][q].x + (double)s_tot[threadIdx.x][q].y;
   if (SH) {
 #pragma unroll
     for (int q = 0; q < NQ; ++q) cv.xs[(int64_t)i * NQ + q] = tot[q];
@@ -1200,7 +1206,7 @@ __global__ void __launch_bounds__(32 * MOM_WARPS) k_moments_wp(CaseView cv, cons
 }
 
 int launch_moments(const CaseView& cv, const void* f, cudaStream_t s) {
-  const int gp = moments_gp(cv.n), W = MOM_WARPS, grid = (cv.n + W * gp - 1) / (W * gp);
+  const int gp = moments_gp(cv.n), W = moments_warps(cv.n), grid = (cv.n + W * gp - 1) / (W * gp);
   const bool row = cv.nv % 4 == 0;
 #define BGK_MOM_WP(S, D)                                                                               \
   {                                                                                                    \
@@ -1299,7 +1305,7 @@ int launch_shard_walls(const CaseView& cv, int phase, cudaStream_t s) {
 }
 
 int launch_shard_partial(const CaseView& cv, cudaStream_t s) {
-  const int gp = moments_gp(cv.n), W = MOM_WARPS, grid = (cv.n + W * gp - 1) / (W * gp);
+  const int gp = moments_gp(cv.n), W = moments_warps(cv.n), grid = (cv.n + W * gp - 1) / (W * gp);
   const bool row = cv.nv % 4 == 0;
 #define BGK_PART_WP(S, D)                                                                                   \
   {                                                                                                         \
