@@ -1370,14 +1370,16 @@ int launch_shard_allreduce(double* const* bufs, int nbufs, int64_t count, cudaSt
 }
 
 // Copies between the caller's dense layout and the padded storage, converting the element
-// type.  Both are bound by HBM.  Without padding (NV % 4 == 0) the arrays are flat: 4
-// elements per thread and access, four accesses in flight (16-byte loads and stores in
-// FP32; pointers aligned to 4 elements).  Otherwise a warp takes whole rows, so that every
-// access of 32 neighbouring elements is contiguous whatever the row's alignment and no
-// thread divides.  One element per thread with a 64-bit division each took 78 us for the
-// 133^2 x 27^2 FP32 state (206 MB moved) and 35 us for 101^2 x 24^2 (94 MB); a pass of the
-// first (two steps and the read-back) takes 419 us instead of 462, the adjoint gradient of
-// 8 steps of the second (with its 21 moment passes) 4.49 ms instead of 4.96.
+// type.  Both are bound by HBM.
+//   Without padding (NV % 4 == 0) the arrays are flat: 4 elements per thread and access, four
+// accesses in flight (16-byte loads and stores in FP32; pointers aligned to 4 elements):
+// 101^2 x 24^2 FP32 (94 MB) 11 us, 33 us with one element per thread and a 64-bit division.
+//   Rows of 256 elements and more: a warp takes whole rows, so that every access of 32
+// neighbouring elements is contiguous whatever the row's alignment, eight of them in flight
+// and no thread divides: 133^2 x 27^2 FP32 (206 MB) 40 us, 82 us by elements with a division.
+//   Shorter rows leave a warp fewer than eight accesses: a CTA takes the elements of a block
+// of whole destination rows in turn and steps through them by additions: 301^2 x 13^2 39 us
+// (69 us by rows), 201^2 x 5^2 2 us less than by rows.
 template <typename A, typename B>
 __global__ void __launch_bounds__(256) k_convert_flat(const A* __restrict__ src, B* __restrict__ dst, int64_t n4) {
   using CA = decltype(ld1(src));
@@ -1410,14 +1412,47 @@ __global__ void __launch_bounds__(256) k_convert_rows(const A* __restrict__ src,
   }
 }
 
+constexpr int kShortRow = 256;       // elements of a row from which it is copied by a warp
+constexpr int kConvertTile = 4096;   // elements of a block of shorter rows
+template <typename A, typename B, bool PAD>
+__global__ void __launch_bounds__(256) k_convert_short(const A* __restrict__ src, B* __restrict__ dst, int64_t rows,
+                                                      int NV, int ls, int ld, int per, int dk, int dsrc) {
+  using CB = decltype(ld1(dst));
+  const int64_t r0 = (int64_t)blockIdx.x * per;
+  const int m = (int)min((int64_t)per, rows - r0) * ld;
+  const int q = fdiv_small(threadIdx.x, 1.0f / (float)ld);
+  int k = threadIdx.x - q * ld;  // position in the row
+  const A* a = src + r0 * ls + q * ls + k;
+  B* b = dst + r0 * ld + threadIdx.x;
+  for (int t = threadIdx.x; t < m; t += 8 * 256, b += 8 * 256) {
+    CB v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      if (t + u * 256 < m) v[u] = !PAD || k < NV ? (CB)ld1(a) : (CB)0;
+      k += dk;
+      a += dsrc;
+      if (k >= ld) { k -= ld; a += ls - ld; }
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (t + u * 256 < m) st1(b + u * 256, v[u]);
+  }
+}
+
 template <typename A, typename B>
 static void convert(const A* src, B* dst, int64_t rows, int NV, int ls, int ld, cudaStream_t s) {
   if (ls == ld && NV == ls && reinterpret_cast<uintptr_t>(src) % (4 * sizeof(A) < 16 ? 4 * sizeof(A) : 16) == 0 &&
       reinterpret_cast<uintptr_t>(dst) % (4 * sizeof(B) < 16 ? 4 * sizeof(B) : 16) == 0) {
     const int64_t n4 = rows * ls / 4;  // (NV is a multiple of 4 here: ls = ld = NV is the padded length)
-    k_convert_flat<<<(int)std::min<int64_t>((n4 + 1023) / 1024, 152 * 32), 256, 0, s>>>(src, dst, n4);
+    k_convert_flat<<<(int)std::min<int64_t>((n4 + 1023) / 1024, TARGET_SMS * 32), 256, 0, s>>>(src, dst, n4);
+  } else if (ld >= kShortRow) {
+    k_convert_rows<<<(int)std::min<int64_t>((rows + 7) / 8, TARGET_SMS * 64), 256, 0, s>>>(src, dst, rows, NV, ls, ld);
   } else {
-    k_convert_rows<<<(int)std::min<int64_t>((rows + 7) / 8, 152 * 64), 256, 0, s>>>(src, dst, rows, NV, ls, ld);
+    // a step of 256 elements: 256 / ld rows and dk elements on (one row more where dk wraps)
+    const int per = kConvertTile / ld, dk = 256 % ld, dsrc = 256 / ld * ls + dk;
+    const int grid = (int)((rows + per - 1) / per);
+    if (ld > NV) k_convert_short<A, B, true><<<grid, 256, 0, s>>>(src, dst, rows, NV, ls, ld, per, dk, dsrc);
+    else k_convert_short<A, B, false><<<grid, 256, 0, s>>>(src, dst, rows, NV, ls, ld, per, dk, dsrc);
   }
 }
 

@@ -36,8 +36,8 @@ constexpr int kMirrorUnroll = 5;
 // With ROW4 (nv % 4 == 0) a lane's 4 velocities share (v_y, v_z), so the
 // projection c.P_d costs one FMA per velocity: c.P_d = c_x P_dx + (c_y P_dy + c_z P_dz).
 // ---------------------------------------------------------------------------
-// Quotient k / n for 0 <= k < 2^13, 1 <= n <= 64 by a float reciprocal: (k + 1/2)/n lies at least
-// 1/(2n) away from an integer and the float error is below (k/n + 1) 2^-23, so truncation is exact.
+// Quotient k / n for 0 <= k < 2^13, 1 <= n <= 2^13 by a float reciprocal: (k + 1/2)/n lies at least
+// 1/(2n) away from an integer and the float error is below (k/n + 1) 2^-22, so truncation is exact.
 __device__ __forceinline__ int fdiv_small(int k, float inv_n) { return (int)(((float)k + 0.5f) * inv_n); }
 
 // Velocity components of the VPL velocities k0..k0+VPL-1.  With ROW (nv % VPL == 0,
