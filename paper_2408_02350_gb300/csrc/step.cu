@@ -1120,13 +1120,14 @@ __global__ void k_moments(CaseView cv, const S* f) {
 // the raw sums of the velocity slab (in FP64) to the exchange buffer instead.  48 registers
 // (5 CTAs per SM), chosen so that the loads of a chunk stay in flight (left to the compiler,
 // 40 for BF16: 35 against 29 us, 41^2 x 63^2).
-constexpr int MOM_GP = 8, MOM_WARPS = 8;  // points per warp, warps per CTA (at most)
-// Points per warp: MOM_GP where that still gives every SM 32 warps, fewer for smaller
-// clouds (8 points per warp left 8 warps per SM on 101^2 points: 32 us for 47 MB).
+constexpr int MOM_GP = 4, MOM_WARPS = 8;  // points per warp, warps per CTA (at most)
+// Points per warp: MOM_GP (32 points per CTA, one full warp of FP64 work) where that still
+// gives every SM 32 warps, fewer for smaller clouds; 8 left the last CTAs uneven (201^2 x
+// 32^2, upload and moments: 161 us, 166 with 32-point CTAs of 4 warps).
 static int moments_gp(int n) { return std::max(1, std::min(MOM_GP, n / (TARGET_SMS * 32))); }
 // Warps per CTA: 8, so that the FP64 part serves 8 points or more at once (21^3 points x 3^3
-// velocities, upload and moments: 17 us; 39 us with a warp for each point's FP64 part, 19 us
-// with 8 points per warp); 4 where the warps do not fill the SMs and 8 would spread them
+// velocities, upload and moments: 17 us; 39 us with a warp for each point's FP64 part, 20 us
+// with 4 warps of 8 points); 4 where the warps do not fill the SMs and 8 would spread them
 // unevenly.
 static int moments_warps(int n) { return n < TARGET_SMS * 32 ? MOM_WARPS / 2 : MOM_WARPS; }
 template <typename S, int DIM, bool ROW, bool SH = false>
@@ -1379,7 +1380,8 @@ int launch_shard_allreduce(double* const* bufs, int nbufs, int64_t count, cudaSt
 // and no thread divides: 133^2 x 27^2 FP32 (206 MB) 40 us, 82 us by elements with a division.
 //   Shorter rows leave a warp fewer than eight accesses: a CTA takes the elements of a block
 // of whole destination rows in turn and steps through them by additions: 301^2 x 13^2 39 us
-// (69 us by rows), 201^2 x 5^2 2 us less than by rows.
+// (69 us by rows), 201^2 x 5^2 7 us (9 us).  Elements past the end load the first one, so
+// that no load waits for a branch.
 template <typename A, typename B>
 __global__ void __launch_bounds__(256) k_convert_flat(const A* __restrict__ src, B* __restrict__ dst, int64_t n4) {
   using CA = decltype(ld1(src));
@@ -1428,7 +1430,9 @@ __global__ void __launch_bounds__(256) k_convert_short(const A* __restrict__ src
     CB v[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      if (t + u * 256 < m) v[u] = !PAD || k < NV ? (CB)ld1(a) : (CB)0;
+      const bool on = t + u * 256 < m && (!PAD || k < NV);
+      v[u] = (CB)ld1(on ? a : src);
+      if (PAD && !on) v[u] = (CB)0;
       k += dk;
       a += dsrc;
       if (k >= ld) { k -= ld; a += ls - ld; }
