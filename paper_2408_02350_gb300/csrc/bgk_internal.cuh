@@ -124,7 +124,19 @@ struct CaseView {
   // second-order step: the state at the start of the step, averaged into the second
   // transport stage (null otherwise)
   void* f_avg;
+  int32_t list3;  // 3D, FP32/BF16: neighbours of a point that its warp stages (staged_nbrs3)
+  int32_t pad_l3;
 };
+
+// Entries of the staged neighbour list of a 3D point for lists of up to cap (max_nbrs).  Lists
+// are sized with room to spare, 160 for about 80 neighbours, and shared memory for all of it
+// would leave 32 KB of L1 for the neighbour rows: 96 for up to 160.  Longer lists are declared
+// for points with well over 96 neighbours, whose reads from global memory cost more than the
+// L1: 160 (25^3 points of about 150 neighbours in lists of 240, us per step with 96 / 160
+// entries: 12^3 velocities 1390 / 1118, BF16 1481 / 1245, ALE 1946 / 1687, 13^3 3158 / 2734;
+// of about 80 in such lists: 546 / 548, 600 / 599, 791 / 811, 1262 / 1280; 128 entries take
+// 1200, 1322, 1798 and 2975 us for the long ones).
+__host__ __device__ constexpr int staged_nbrs3(int cap) { return cap > 160 ? 160 : (cap > 96 ? 96 : cap); }
 
 // The derived per-case constants of CaseView (wv, h2 and the FP32 copies), from dim, dt,
 // kn, dv, h, alpha.
@@ -137,6 +149,7 @@ inline void set_case_consts(CaseView& v) {
   v.two_dt_f = (float)(2.0 * v.dt);
   v.kn_f = (float)v.kn;
   v.wv_f = (float)v.wv;
+  v.list3 = staged_nbrs3(v.cap);
 }
 
 // Launchers (stream-ordered; each returns the number of kernels launched).

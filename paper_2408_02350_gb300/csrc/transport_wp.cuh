@@ -506,16 +506,12 @@ __device__ __forceinline__ void ks_load(const float* s_k, const int lane, float 
 // The point's list and stencil in the warp's shared memory.  2D: the indices, then one
 // 16-byte entry per neighbour.  3D: one 48-byte entry per neighbour, rows (P_dx, P_dy,
 // P_dz, .) with the neighbour's index in the first spare word, so that a neighbour costs
-// three 16-byte loads instead of ten 4-byte ones; only the first kList3 neighbours are
-// staged (max_nbrs is sized for dense clouds, 160 for about 80 neighbours, and shared
-// memory for all of it would leave 32 KB of L1 for the neighbour rows); the rest are read
-// from global memory.  With 4-byte entries for all of max_nbrs and 64-bit row indices the
-// 41^3 x 16^3 transport took 5.97 ms per launch (4.96 now), 27^3 x 12^3 ALE 1042 us (834).
-constexpr int kList3 = 96;
+// three 16-byte loads instead of ten 4-byte ones; only the first cv.list3 neighbours are
+// staged (staged_nbrs3); the rest are read from global memory, one at a time.  With 4-byte
+// entries for all of max_nbrs and 64-bit row indices the 41^3 x 16^3 transport took 5.97 ms
+// per launch (4.96 now), 27^3 x 12^3 ALE 1042 us (834).
 template <int DIM>
-__host__ __device__ constexpr int staged_nbrs(int cap) { return DIM == 3 && cap > kList3 ? kList3 : cap; }
-template <int DIM>
-__host__ __device__ constexpr int list_floats(int cap) { return DIM == 3 ? 12 * staged_nbrs<3>(cap) : 5 * cap; }
+__host__ __device__ constexpr int list_floats(int cap) { return DIM == 3 ? 12 * staged_nbrs3(cap) : 5 * cap; }
 
 template <int DIM>
 __device__ __forceinline__ void stage_list(const CaseView& cv, const int i, const int m, float* s_P, int32_t* s_col) {
@@ -526,7 +522,7 @@ __device__ __forceinline__ void stage_list(const CaseView& cv, const int i, cons
     for (int q = lane; q < m; q += 32) s_col[q] = checked_index(col[q], cv.n, i, cv.status);
     for (int q = lane; q < m * 4; q += 32) s_P[q] = P[q];
   } else {
-    const int ms = min(m, kList3);
+    const int ms = min(m, cv.list3);
     for (int q = lane; q < ms; q += 32) s_P[12 * q + 3] = __int_as_float(checked_index(col[q], cv.n, i, cv.status));
     for (int q = lane; q < ms * 9; q += 32) {
       const int e = q / 9, r = q - 9 * e;
@@ -572,7 +568,7 @@ __device__ __forceinline__ void transport_point_wp(const CaseView& cv, const int
   const int m = checked_count(cv.cnt[i], cap, cv.status);
   for (int q = lane; q < nv; q += 32) s_v[q] = cv.vnodes_f[q];
   stage_list<DIM>(cv, i, m, s_P, s_col);
-  const int ms = DIM == 3 ? min(m, kList3) : m;  // staged neighbours
+  const int ms = DIM == 3 ? min(m, cv.list3) : m;  // staged neighbours
   __syncwarp();
 
   float U[DIM];
@@ -749,7 +745,7 @@ __device__ __forceinline__ void transport_point_mirror(const CaseView& cv, const
   const int m = checked_count(cv.cnt[i], cap, cv.status);
   for (int q = lane; q < nv; q += 32) s_v[q] = cv.vnodes_f[q];
   stage_list<DIM>(cv, i, m, s_P, s_col);
-  const int ms = DIM == 3 ? min(m, kList3) : m;  // staged neighbours
+  const int ms = DIM == 3 ? min(m, cv.list3) : m;  // staged neighbours
   __syncwarp();
 
   const int nchunk = NV / (2 * VPL);
