@@ -121,7 +121,7 @@ struct bgk_ctx {
   CaseView* d_cases[2] = {nullptr, nullptr};
   int2* d_items = nullptr;
   int2* d_witems = nullptr;
-  int n_items = 0, n_witems = 0, capmax = 0, nvpmax = 0, batch_dim = 0, batch_storage = 0;
+  int n_items = 0, n_witems = 0, capmax = 0, nvpmax = 0, batch_storage = 0;
   // (4 warps per CTA: 1409 us per step of 24 cavities of up to 121^2 points, 1432 with 8)
   int batch_warps = 4, batch_grid = 0;
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
@@ -492,7 +492,6 @@ int prepare_batch(bgk_ctx* ctx, cudaStream_t s) {
     ctx->n_items = (int)items.size();
     ctx->n_witems = (int)witems.size();
     ctx->capmax = capmax;
-    ctx->batch_dim = ctx->cases[0].cv.dim;
     ctx->batch_storage = ctx->cases[0].p.storage;
   }
   std::vector<CaseView> views(nc);
@@ -511,10 +510,10 @@ int prepare_batch(bgk_ctx* ctx, cudaStream_t s) {
 }
 
 int launch_batch_step(bgk_ctx* ctx, int parity, cudaStream_t s) {
-  ctx->launches += launch_transport_batch(ctx->d_cases[parity], ctx->d_items, ctx->n_items, ctx->batch_dim,
-                                          ctx->batch_storage, ctx->capmax, ctx->batch_warps, ctx->batch_grid, s);
-  ctx->launches += launch_walls_batch(ctx->d_cases[parity], ctx->d_witems, ctx->n_witems, ctx->batch_dim,
-                                      ctx->batch_storage, ctx->capmax, ctx->nvpmax, s);
+  ctx->launches += launch_transport_batch(ctx->d_cases[parity], ctx->d_items, ctx->n_items, ctx->batch_storage,
+                                          ctx->capmax, ctx->batch_warps, ctx->batch_grid, s);
+  ctx->launches += launch_walls_batch(ctx->d_cases[parity], ctx->d_witems, ctx->n_witems, ctx->batch_storage,
+                                      ctx->capmax, ctx->nvpmax, s);
   CKL(ctx);
   return BGK_OK;
 }
@@ -1590,8 +1589,8 @@ int bgk_autotune(bgk_ctx* ctx, void* stream) {
       // the transport launch reads f_in and writes f_out only, so repeating it leaves the state unchanged
       for (int rep = 0; rep < 6; ++rep) {
         if (rep == 1) cudaEventRecord(e0, s);
-        ctx->launches += launch_transport_batch(ctx->d_cases[parity], ctx->d_items, ctx->n_items, ctx->batch_dim,
-                                                ctx->batch_storage, ctx->capmax, warps_c[wi], grid, s);
+        ctx->launches += launch_transport_batch(ctx->d_cases[parity], ctx->d_items, ctx->n_items, ctx->batch_storage,
+                                                ctx->capmax, warps_c[wi], grid, s);
       }
       cudaEventRecord(e1, s);
       CKL(ctx);

@@ -210,10 +210,10 @@ int launch_transport_f64_avg(const CaseView& cv, cudaStream_t s);
 int launch_relax_half_f64(const CaseView& cv, cudaStream_t s);
 int launch_shard_relax_f64(const CaseView& cv, cudaStream_t s);
 int launch_walls(const CaseView& cv, cudaStream_t s);
-// Batched (many cases, one launch each): FP32/BF16 storage, all cases of one dimension.
-int launch_transport_batch(const CaseView* d_cases, const int2* items, int n_items, int dim, int storage, int capmax,
+// Batched (many cases, one launch each): 2D cases of one storage type, FP32 or BF16.
+int launch_transport_batch(const CaseView* d_cases, const int2* items, int n_items, int storage, int capmax,
                            int warps, int grid, cudaStream_t s);
-int launch_walls_batch(const CaseView* d_cases, const int2* witems, int n_witems, int dim, int storage, int capmax,
+int launch_walls_batch(const CaseView* d_cases, const int2* witems, int n_witems, int storage, int capmax,
                        int nvpmax, cudaStream_t s);
 int launch_move(const CaseView& cv, cudaStream_t s);
 int launch_set_maxwellian(const CaseView& cv, double rho0, const double* u0, double T0, cudaStream_t s);

@@ -28,10 +28,6 @@ namespace bgk {
 
 static inline int grid_for(int64_t n, int block) { return (int)((n + block - 1) / block); }
 
-// Fixed points: pair each velocity with its mirror in the transport (1) or not (0).
-#ifndef BGK_TRANSPORT_MIRROR
-#define BGK_TRANSPORT_MIRROR 1
-#endif
 __host__ __device__ static inline size_t align16(size_t b) { return (b + 15) & ~size_t(15); }
 
 constexpr int RED_BYTES = 32 * 8 * 8;   // block-reduction scratch: 8 values x 32 warps, double
@@ -222,38 +218,39 @@ __global__ void __launch_bounds__(256) k_shard_relax_wp(const CaseView cv) {
 // warp per interior point, each lane a velocity chunk and its mirror chunk; 128 registers,
 // 16 warps per SM, five neighbours' rows in flight per warp (24 warps with 80 registers and
 // two or three neighbours: 5.36 / 5.33 against 4.96 ms, 41^3 x 16^3).  Used in 3D, where it
-// saves a quarter of the per-neighbour instructions; in 2D the extra registers cost more
-// than the saved instructions (201^2 x 32^2 fixed points: 0.483 ms at 4 CTAs per SM with
-// spills, 0.561 ms at 3, against 0.447 ms), so 2D keeps the plain kernel.
-template <typename S, int DIM, bool KS>
+// saves a quarter of the per-neighbour instructions; in 2D the extra registers cost about
+// what the instructions save, and more in smaller clouds, so 2D keeps the plain kernel: step
+// of 201^2 x 32^2 fixed points FP32 0.410 ms, paired 0.412 / 0.421 with 16 warps per SM and 5
+// / 3 neighbours, 0.409 / 0.404 with 24 and 3 / 2, 0.438 with 32 and 2; 101^2 x 24^2 0.088
+// against 0.094 ms at best (BF16 201^2 x 32^2: 0.423, paired 0.396 with 16 warps).
+template <typename S, int DIM>
 __global__ void __launch_bounds__(256, 2) k_transport_mirror(const CaseView cv) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int W = blockDim.x >> 5, warp = threadIdx.x >> 5;
   const WarpShared<DIM> ws(smem, W, warp, cv.cap);
   const int t = blockIdx.x * W + warp;
   if (t >= cv.n_int) return;
-  transport_point_mirror<S, DIM, KS>(cv, cv.int_idx[t], ws.v, ws.col, ws.P, ws.k);
+  transport_point_mirror<S, DIM>(cv, cv.int_idx[t], ws.v, ws.col, ws.P);
 }
 
 // Many cases in one persistent launch: items[k] = (case, interior slot), tiles of W
 // consecutive items per CTA, tiles taken in grid-stride order.  Every warp reads
 // its case's descriptor; the ROW4 variant is chosen per warp.
-// 3 CTAs per SM (80 registers, 8 bytes spilled) beats 2 (114 registers, no spills) on
-// the 64-cavity sweep: 4.54 against 4.99 ms per step (when measured); the compensated
-// sums in shared memory (KS, as the single-case kernel) lose here: 4.46 ms at 3 CTAs per
-// SM and 4.57 ms at 4 against 4.04 ms.
+// 80 registers, 24 warps per SM (launched with 4 warps per CTA): a step of 24 cavities of up
+// to 121^2 points takes 1409 us, 1743 with 16 warps, 1464 to 1580 with the compensated sums
+// in shared memory (KS, as the single-case kernel), 1432 with 8 warps per CTA.
 #ifndef BGK_BATCH_KS
 #define BGK_BATCH_KS false
 #endif
 #ifndef BGK_BATCH_MIN_BLOCKS
 #define BGK_BATCH_MIN_BLOCKS 3
 #endif
-template <typename S, int DIM>
+template <typename S>
 __global__ void __launch_bounds__(256, BGK_BATCH_MIN_BLOCKS) k_transport_batch(const CaseView* __restrict__ cases, const int2* __restrict__ items,
                                                              int n_items, int capmax) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int W = blockDim.x >> 5, warp = threadIdx.x >> 5;
-  const WarpShared<DIM> ws(smem, W, warp, capmax);
+  const WarpShared<2> ws(smem, W, warp, capmax);
   for (int tile = blockIdx.x; tile * W < n_items; tile += gridDim.x) {
     const int it = tile * W + warp;
     if (it >= n_items) continue;
@@ -261,37 +258,35 @@ __global__ void __launch_bounds__(256, BGK_BATCH_MIN_BLOCKS) k_transport_batch(c
     const CaseView& cv = cases[e.x];
     const int i = cv.int_idx[e.y];
     // (batched stepping takes fixed points only: c = v)
-    if (cv.nv % 4 == 0) transport_point_wp<S, DIM, false, true, 4, BGK_BATCH_KS>(cv, i, ws.v, ws.col, ws.P, ws.k);
-    else transport_point_wp<S, DIM, false, false, 4, BGK_BATCH_KS>(cv, i, ws.v, ws.col, ws.P, ws.k);
+    if (cv.nv % 4 == 0) transport_point_wp<S, 2, false, true, 4, BGK_BATCH_KS>(cv, i, ws.v, ws.col, ws.P, ws.k);
+    else transport_point_wp<S, 2, false, false, 4, BGK_BATCH_KS>(cv, i, ws.v, ws.col, ws.P, ws.k);
     __syncwarp();
   }
 }
 
-// Velocities per lane: 8 in 3D when the velocity rows split into groups of 8 (fewer
-// per-neighbour instructions and more loads in flight pay off there: 7.1 vs 8.6 ms
-// on the 41^3 x 16^3 cavity), 4 in 2D (where the lower occupancy of the wider
-// variant costs more than it saves: 0.53 vs 0.48 ms on the 201^2 x 32^2 cavity).
-int transport_vpl = 0;  // 0 = automatic; 4 or 8 forces a width
-
+// Velocities per lane of moving points: 8 in 3D when the velocity rows split into groups of
+// 8, whose rows cost fewer instructions per velocity and keep more loads in flight (first
+// measured on fixed points, 41^3 x 16^3, which take the pairs now: 7.1 against 8.6 ms per
+// step); 4 in 2D, where the lower occupancy of the wider variant costs more than it saves
+// (201^2 x 32^2, at the time: 0.53 against 0.48 ms).
 template <typename S, int DIM>
 static void launch_transport_wp(const CaseView& cv, cudaStream_t s) {
   const int W = BGK_WP_WARPS, threads = 32 * W;
   const size_t smem = wp_smem_bytes<DIM>(W, cv.cap);
   const int grid = (cv.n_int + W - 1) / W;
-  const bool row4 = cv.nv % 4 == 0, row8 = cv.nv % 8 == 0 && cv.NVp % 8 == 0;
+  const bool row4 = cv.nv % 4 == 0;
   if constexpr (DIM == 3) {
-    if (BGK_TRANSPORT_MIRROR && !cv.ale && row4 && cv.NV % 8 == 0) {
-      auto k = k_transport_mirror<S, DIM, false>;
+    if (!cv.ale && row4) {  // (then NV % 8 == 0: the chunks of 4 pair up)
+      auto k = k_transport_mirror<S, DIM>;
       const size_t msm = wp_smem_bytes<DIM>(W, cv.cap, false);
       cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)msm);
       k<<<grid, threads, msm, s>>>(cv);
       return;
     }
   }
-  const bool v8 = transport_vpl == 8 ? (cv.NVp % 8 == 0) : (transport_vpl == 4 ? false : (DIM == 3 && row8));
   if constexpr (BGK_WP_STAGE && DIM == 2 && std::is_same<S, float>::value) {
     // (bulk copies need 16-byte aligned rows: caller-bound storage may start anywhere)
-    if (row4 && !v8 && cv.NVp % 4 == 0 && (reinterpret_cast<uintptr_t>(cv.f_in) & 15) == 0) {
+    if (row4 && cv.NVp % 4 == 0 && (reinterpret_cast<uintptr_t>(cv.f_in) & 15) == 0) {
       const size_t ssm = stage_smem_bytes(smem, W);
       auto k = cv.ale ? k_transport_stage<true> : k_transport_stage<false>;
       cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm);
@@ -305,12 +300,11 @@ static void launch_transport_wp(const CaseView& cv, cudaStream_t s) {
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);       \
     k<<<grid, threads, smem, s>>>(cv);                                                    \
   }
-  if (v8) {
-    if (cv.ale) {
-      if (row8) BGK_LAUNCH_WP(true, true, 8) else BGK_LAUNCH_WP(true, false, 8)
-    } else {
-      if (row8) BGK_LAUNCH_WP(false, true, 8) else BGK_LAUNCH_WP(false, false, 8)
-    }
+  if constexpr (DIM == 3) {
+    if (!cv.ale) BGK_LAUNCH_WP(false, false, 4)
+    else if (cv.nv % 8 == 0) BGK_LAUNCH_WP(true, true, 8)
+    else if (row4) BGK_LAUNCH_WP(true, true, 4)
+    else BGK_LAUNCH_WP(true, false, 4)
   } else if (cv.ale) {
     if (row4) BGK_LAUNCH_WP(true, true, 4) else BGK_LAUNCH_WP(true, false, 4)
   } else {
@@ -758,47 +752,36 @@ __global__ void __launch_bounds__(256) k_walls(const CaseView cv) {
 }
 
 // witems[k] = (case, wall slot): one CTA per wall point of any case
-template <typename S, typename C, int DIM>
+template <typename S, typename C>
 __global__ void __launch_bounds__(256) k_walls_batch(const CaseView* __restrict__ cases, const int2* __restrict__ witems) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int2 e = witems[blockIdx.x];
-  walls_point_v4<S, C, DIM>(cases[e.x], e.y, smem);
+  walls_point_v4<S, C, 2>(cases[e.x], e.y, smem);
 }
 
-int launch_transport_batch(const CaseView* d_cases, const int2* items, int n_items, int dim, int storage, int capmax,
+int launch_transport_batch(const CaseView* d_cases, const int2* items, int n_items, int storage, int capmax,
                            int warps, int grid, cudaStream_t s) {
   if (n_items == 0) return 0;
   const int threads = 32 * warps;
-  const size_t smem = dim == 2 ? wp_smem_bytes<2>(warps, capmax) : wp_smem_bytes<3>(warps, capmax);
+  const size_t smem = wp_smem_bytes<2>(warps, capmax);
   const int ntiles = (n_items + warps - 1) / warps;
   if (grid <= 0 || grid > ntiles) grid = ntiles;
-#define BGK_BATCH(S, D)                                                                    \
-  {                                                                                        \
-    auto k = k_transport_batch<S, D>;                                                      \
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);        \
-    k<<<grid, threads, smem, s>>>(d_cases, items, n_items, capmax);                        \
-  }
-  if (dim == 2) {
-    if (storage == 1) BGK_BATCH(float, 2) else BGK_BATCH(__nv_bfloat16, 2)
-  } else {
-    if (storage == 1) BGK_BATCH(float, 3) else BGK_BATCH(__nv_bfloat16, 3)
-  }
-#undef BGK_BATCH
+  auto go = [&](auto k) {
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k<<<grid, threads, smem, s>>>(d_cases, items, n_items, capmax);
+  };
+  if (storage == 1) go(k_transport_batch<float>);
+  else go(k_transport_batch<__nv_bfloat16>);
   return 1;
 }
 
-int launch_walls_batch(const CaseView* d_cases, const int2* witems, int n_witems, int dim, int storage, int capmax,
+int launch_walls_batch(const CaseView* d_cases, const int2* witems, int n_witems, int storage, int capmax,
                        int nvpmax, cudaStream_t s) {
   if (n_witems == 0) return 0;
   const size_t smem = wall_smem(capmax);
   const int threads = wall_threads(nvpmax);
-  if (dim == 2) {
-    if (storage == 1) k_walls_batch<float, float, 2><<<n_witems, threads, smem, s>>>(d_cases, witems);
-    else k_walls_batch<__nv_bfloat16, float, 2><<<n_witems, threads, smem, s>>>(d_cases, witems);
-  } else {
-    if (storage == 1) k_walls_batch<float, float, 3><<<n_witems, threads, smem, s>>>(d_cases, witems);
-    else k_walls_batch<__nv_bfloat16, float, 3><<<n_witems, threads, smem, s>>>(d_cases, witems);
-  }
+  if (storage == 1) k_walls_batch<float, float><<<n_witems, threads, smem, s>>>(d_cases, witems);
+  else k_walls_batch<__nv_bfloat16, float><<<n_witems, threads, smem, s>>>(d_cases, witems);
   return 1;
 }
 

@@ -447,13 +447,12 @@ void launch_f64(const CaseView& cv, cudaStream_t s) {
     return;
   }
   if constexpr (ROW && !SH) {
-    // the whole grid in chunks of 4 that pair up: v at k, -v at NV - 1 - k
-    if (cv.NV % 8 == 0) {
-      go(k_transport_f64<DIM, ROW, false, SH, AVG, true>, cv.NV / 8);
-      return;
-    }
+    // the whole grid in chunks of 4 that pair up: v at k, -v at NV - 1 - k (nv % 4 == 0, so
+    // NV % 8 == 0)
+    go(k_transport_f64<DIM, ROW, false, SH, AVG, true>, cv.NV / 8);
+  } else {
+    go(k_transport_f64<DIM, ROW, false, SH, AVG, false>, cv.NVp / 4);
   }
-  go(k_transport_f64<DIM, ROW, false, SH, AVG, false>, cv.NVp / 4);
 }
 
 template <bool SH, bool AVG>

@@ -459,14 +459,15 @@ __device__ __forceinline__ void partial_out(const CaseView& cv, const int i, con
 }
 
 // The per-point body, shared by the single-case kernel and the batched kernel:
-// one warp, point i of case cv; s_v, s_col, s_P, s_k are this warp's shared buffers
-// (nv, cap, cap * dim^2 and kahan_floats(DIM) entries).  Each lane owns VPL
+// one warp, point i of case cv; s_v, s_col, s_P, s_k are this warp's shared buffers (64 nodes;
+// 2D: cap indices and cap 16-byte entries, 3D: s_col null and cv.list3 48-byte entries at
+// most; kahan_floats<DIM>() floats, KS only).  Each lane owns VPL
 // consecutive velocities of every (32 VPL)-velocity slice.  With KS the lanes'
 // compensated moment sums live in s_k between slices and the velocities are
 // recomputed after the neighbour loop, which keeps the 4-velocity body within 64
 // registers (32 warps per SM: 0.432 against 0.465 ms with 24 on the 201^2 x 32^2 ALE
-// cavity); without KS they stay in registers (the 8-velocity 3D
-// body and the batched kernel, which lose with KS).  SH (sharded step): the row holds
+// cavity, before the rows were addressed by row_at); without KS they stay in registers (the
+// 8-velocity 3D body and the batched kernel, which lose with KS).  SH (sharded step): the row holds
 // the velocity slab that starts at cv.vk0, and the slab's moment sums of f~ go to the
 // exchange buffer instead of the relaxation.  AVG (second stage of the second-order
 // step): f~ is averaged with the row of cv.f_avg and relaxed exactly over dt/2.
@@ -733,9 +734,9 @@ __device__ __forceinline__ void transport_point_wp(const CaseView& cv, const int
 // so m(-v) of the lane's pair (v_{2q}, v_{2q+1}) is the mirror chunk's pair 1 - q with
 // its halves swapped.  Each neighbour row then costs the projections once for 8
 // velocities.  Requires nv % 4 == 0 and NV % 8 == 0 (then NVp = NV).
-template <typename S, int DIM, bool KS>
+template <typename S, int DIM>
 __device__ __forceinline__ void transport_point_mirror(const CaseView& cv, const int i, float* s_v, int32_t* s_col,
-                                                       float* s_P, float* s_k) {
+                                                       float* s_P) {
   constexpr int NC = DIM == 2 ? 2 : 1;
   constexpr int DD = DIM * DIM;
   constexpr int VPL = 4, NP = 2;
@@ -758,7 +759,6 @@ __device__ __forceinline__ void transport_point_mirror(const CaseView& cv, const
   float rsum[DIM + 2], rcmp[DIM + 2];
 #pragma unroll
   for (int q = 0; q < DIM + 2; ++q) { rsum[q] = 0.0f; rcmp[q] = 0.0f; }
-  if (KS) ks_store<DIM>(s_k, lane, rsum, rcmp);
 
   for (int sl = 0; sl < nslice; ++sl) {
     const int chunk = sl * 32 + lane;
@@ -853,17 +853,8 @@ __device__ __forceinline__ void transport_point_mirror(const CaseView& cv, const
     for (int e = 0; e < VPL; ++e)
 #pragma unroll
       for (int a = 0; a < DIM; ++a) velm[e][a] = -vel[VPL - 1 - e][a];
-    if (KS) {
-      ks_load<DIM>(s_k, lane, rsum, rcmp);
-    }
     slice_out<S, DIM, NC, VPL, false, true>(cv, i, k0, vel, kin, acc, sk, two_dt, rsum, rcmp);
     slice_out<S, DIM, NC, VPL, false, true>(cv, i, km, velm, kin, accm, skm, two_dt, rsum, rcmp);
-    if (KS) {
-      ks_store<DIM>(s_k, lane, rsum, rcmp);
-    }
-  }
-  if (KS) {
-    ks_load<DIM>(s_k, lane, rsum, rcmp);
   }
   finish_point<S, DIM, true, VPL>(cv, i, s_v, rsum, rcmp);
 }
