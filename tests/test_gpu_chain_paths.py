@@ -116,3 +116,44 @@ def test_timeout_on_the_first_step_is_reported_as_such(g, wls, storage):
     assert np.array_equal(s.get_f(), ref.get_f()) and np.array_equal(s.positions(), ref.positions())
     s.close()
     ref.close()
+
+
+# Second-order stencils on moving points: lists from the side chain, the fit after it.  FP32
+# within the project's 1e-4; BF16 rounds f once per step to 2^-9, so three steps are within
+# 3 x 2^-9 of rho and T (6e-3) even if every rounding had the same sign.
+@pytest.mark.parametrize("dim,n,nv,storage,body,steps,tol", [
+    (3, 9, 6, "f32", False, 6, 1e-4), (3, 9, 8, "f32", False, 6, 1e-4), (3, 9, 6, "bf16", False, 3, 6e-3),
+    (2, 21, 8, "bf16", False, 3, 6e-3), (2, 21, 7, "bf16", False, 3, 6e-3), (2, 41, 8, "f32", True, 8, 1e-4)])
+def test_second_order_stencils_of_moving_points(g, dim, n, nv, storage, body, steps, tol):
+    import oracle
+    name = "body2d_ale_n201_v32_f32" if body else "cavity2d_n41_v16_f64" if dim == 2 else "cavity3d_n41_v16_f32"
+    p = bi.config(name, n=n, nv=nv, vmax=4.0, storage=storage, ale=1, wls_order=2)
+    cl = bi.cloud_for(p)
+    sim = oracle.Simulation(p, cl)
+    sim.run(steps)
+    s = g.Solver([p], [cl])
+    s.set_maxwellian()
+    s.step(steps)
+    s.sync()
+    rho, u, T = s.moments()
+    x = s.positions()
+    s.close()
+    assert np.abs(rho - sim.rho).max() < tol * np.abs(sim.rho).max() and np.abs(T - sim.T).max() < tol * np.abs(sim.T).max()
+    if storage == "f32":
+        assert np.abs(u - sim.U).max() < tol * np.abs(sim.U).max() and np.abs(x - sim.x).max() < 1e-6
+
+
+def test_second_order_stencils_of_moving_points_in_slabs(g):
+    # two velocity slabs of the same case, the same bar against the oracle
+    import oracle
+    from paper_2408_02350_gb300.sharded import ShardedSolver
+    p = _ale(wls_order=2)
+    cl = bi.cloud_for(p)
+    sim = oracle.Simulation(p, cl)
+    sim.run(6)
+    s = ShardedSolver.on_one_device(p, cl, 2)
+    s.set_maxwellian()
+    s.step(6)
+    s.sync()
+    rho, u, T = s.moments()
+    assert np.abs(rho - sim.rho).max() < 1e-4 and np.abs(u - sim.U).max() < 1e-4 and np.abs(T - sim.T).max() < 1e-4
