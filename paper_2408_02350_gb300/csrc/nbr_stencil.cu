@@ -306,9 +306,8 @@ __device__ void wall_recon_point(const CaseView& cv, const double* xi, const int
 // that the coefficients will take, the elimination goes down only (rows swapped by
 // selects, so everything stays in registers) with one reciprocal per pivot, and the
 // frames need no square root: P_d = e_d (e_d.coef) = d (d.coef) / r^2 with d = dr for the
-// normal and d = (-dr_y, dr_x) for the tangent.  181^2 points, 24^2 velocities, two ALE
-// steps: 1083 us with the square matrix in local memory, every weight computed twice and
-// full elimination (281 us of each step), 816 us now.
+// normal and d = (-dr_y, dr_x) for the tangent.  181^2 points: 167 us per launch, 281 us with
+// the square matrix in local memory, every weight computed twice and full elimination.
 template <typename C>
 __device__ __forceinline__ void quad_stencil_2d(const CaseView& cv, const int i, const double* xi, const int32_t* row,
                                                 const int m, C* P) {

@@ -17,9 +17,9 @@
 //     the four moment sums are reduced across the warp transposed.
 // f~ goes to the output row and is read back from there for the relaxation, so a thread
 // takes any number of velocity chunks.
-// 41^2 points x 16^2 velocities, fixed points, two steps and the moments: 486 us per pass
-// before (c.P_d in full per velocity, FP64 comparisons, one exponential per velocity),
-// 247 us now.
+// 41^2 points x 16^2 velocities, fixed points: 104 us per launch with the FP64 pipe 84 %
+// busy (221 us with c.P_d in full per velocity, FP64 comparisons and one exponential per
+// velocity).
 #include <algorithm>
 
 #include "bgk_internal.cuh"
@@ -152,8 +152,8 @@ __device__ __forceinline__ void cta_totals(F64Shared& sm, double (&s)[N], double
 
 // Moments from the raw sums, tau and the relaxation of the output row (which holds f~):
 // f^{n+1} = (tau f~ + dt M)/(tau + dt), or with RK = 1 the exact relaxation over dt/2.
-// Every thread forms the moments (the FP64 pipe works per warp, so one thread would cost
-// the same).  The row starts at grid velocity vk0.
+// The lanes of the first warp form the moments, each the same (the FP64 pipe works per warp,
+// so one lane would cost the same).  The row starts at grid velocity vk0.
 template <int DIM, bool ROW, int RK>
 __device__ __forceinline__ void relax_f64(const CaseView& cv, F64Shared& sm, const int i, const double (&tot)[DIM + 2],
                                           const int vk0) {

@@ -12,14 +12,17 @@ namespace bgk {
 // measured with the row addresses of row_at: the kernels wait for rows that miss L1 (long
 // scoreboard), so more rows in flight pay until the registers cost a CTA per SM.
 //   2D, shared grid row per lane: 4 (201^2 x 32^2 ALE: 1 / 2 / 3 / 4 rows 487 / 410 / 419 /
-//   406 us per launch; BF16 469 / 447 / 445 / 432);
-//   2D, ragged velocity grids: 2 (133^2 x 27^2: 173 us; 1 / 3 / 4 rows 192 / 196 / 190);
+//   406 us per launch; BF16 469 / 447 / 445 / 432; per step with 2 / 4 rows: 301^2 x 24^2 ALE
+//   652 / 647, 161^2 x 20^2 fixed 152 / 150, 101^2 x 24^2 fixed 92 / 91);
+//   2D, ragged velocity grids: 2 (133^2 x 27^2: 173 us; 1 / 3 / 4 rows 192 / 196 / 190; per
+//   step with 2 / 4 rows: 301^2 x 21^2 552 / 587, 101^2 x 25^2 105 / 115);
 //   3D: 2 (27^3 x 12^3 ALE: 1 / 2 / 3 / 4 rows 944 / 834 / 847 / 834 us);
 //   mirror pairs (two rows per neighbour): 5 at 16 warps per SM (41^3 x 16^3: 2 / 4 / 5 / 6
 //   / 8 neighbours 5.76 / 5.07 / 4.96 / 5.00 / 4.98 ms; 5.33 ms at best with 24 warps).
 //   2D, shared grid row, a slab of the velocity grid in FP32: 2 (step of the 201^2 x 32^2
 //   ALE case in 1 slab: 1 / 2 / 3 / 4 rows 0.620 / 0.543 / 0.566 / 0.556 ms; in 4 slabs
-//   0.954 / 0.885 / 0.909 / 0.901); BF16 keeps 4 (2 slabs: 0.688 / 0.648 / 0.652 / 0.639).
+//   0.954 / 0.885 / 0.909 / 0.901; 301^2 x 24^2 ALE, 2 slabs, 2 / 4 rows 1.059 / 1.081, fixed
+//   points 161^2 x 32^2, 4 slabs, 0.547 / 0.545); BF16 keeps 4 (2 slabs: 0.688 / 0.648 / 0.652 / 0.639).
 template <typename S, int DIM, bool ROW, bool SH>
 __host__ __device__ constexpr int nbr_unroll() {
   return DIM == 2 && ROW && !(SH && sizeof(S) == 4) ? 4 : 2;
@@ -664,7 +667,9 @@ __device__ __forceinline__ void transport_point_wp(const CaseView& cv, const int
         float fv[NC][VPL];
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
-          // (2D: 64-bit indices here; row_at took 190 against 173 us, 133^2 x 27^2)
+          // (2D: 64-bit indices here.  row_at took 190 against 173 us, 133^2 x 27^2 fixed
+          // points; per step 117 / 105, 101^2 x 25^2, and 605 / 552, 301^2 x 21^2; ALE 201^2 x
+          // 30^2 576 / 578)
           if constexpr (DIM == 2) ldv_ro<S, VPL>(fj0 + (int64_t)j * rowlen + (int64_t)c * NVp, fv[c]);
           else ldv_ro<S, VPL>(row_at(fj0, j, rb), fv[c]);
         }
