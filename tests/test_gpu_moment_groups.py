@@ -1,8 +1,9 @@
 """The moments that bgk_set_f takes, at every number of points per warp (1, 2 and 4 by the size
-of the cloud) and of warps per CTA, with clouds that leave the last CTA partly filled: rho, U and T of every
-point against FP64 sums of the stored values.  The kernel rounds a term at most six times in
-FP32 (node, products, sums of four) and compensates the rest, so a sum is within 6 x 2^-24 of
-the sum of its terms' magnitudes: 1e-6 for rho, 3e-6 for U (mean |v| below 3) and T."""
+of the cloud) and of warps per CTA, with clouds that leave the last CTA partly filled: rho, U
+and T of every point against FP64 sums of the stored values.  The kernel rounds a term at most
+six times in FP32 (node, products, sums of four) and compensates the rest, so a sum is within
+6 x 2^-24 of the sum of its terms' magnitudes: 1e-6 for rho, 3e-6 for U (mean |v| below 3) and
+T."""
 import numpy as np
 import pytest
 
